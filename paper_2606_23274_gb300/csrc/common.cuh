@@ -145,6 +145,18 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+// Pair k of a round of the circle method over P columns (P even).
+__device__ __forceinline__ void rr_pair(int round, int k, int P, int& i, int& j) {
+  const int n = P - 1;
+  if (k == 0) {
+    i = 0;
+    j = 1 + round % n;
+  } else {
+    i = 1 + (round + k) % n;
+    j = 1 + (round - k + n) % n;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon et al., SC'11) and the Box-Muller Gaussian of element
 // i of stream s: counter (i lo, i hi, s lo, s hi), key (seed lo, seed hi);

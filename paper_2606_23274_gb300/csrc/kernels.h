@@ -74,6 +74,11 @@ template <typename C, typename S>
 cudaError_t jacobi_svd(int q, int p, S* W, S* U, S* Sv, S* V, S* Vwork, int max_sweeps, uint32_t* errw,
                        cudaStream_t st);
 
+// The FP64 decomposition on a cluster (jacobi64.cu), which jacobi_svd takes where it
+// fits; cudaErrorNotSupported otherwise. W is not changed.
+cudaError_t jacobi_svd64(int q, int p, const double* W, double* U, double* Sv, double* V, int max_sweeps,
+                         uint32_t* errw, cudaStream_t st);
+
 // ||X||_F of n values (type T) into *out (double), flags non-finite values.
 template <typename T>
 cudaError_t frob_norm(const T* x, long long n, double* out, uint32_t* errw, cudaStream_t st);

@@ -782,17 +782,6 @@ template cudaError_t qr_householder<float, float>(int, int, float*, float*, floa
 // round applies P/2 disjoint plane rotations that orthogonalise column pairs;
 // a sweep is P-1 rounds; it stops after a sweep without rotations.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void rr_pair(int round, int k, int P, int& i, int& j) {
-  const int n = P - 1;
-  if (k == 0) {
-    i = 0;
-    j = 1 + round % n;
-  } else {
-    i = 1 + (round + k) % n;
-    j = 1 + (round - k + n) % n;
-  }
-}
-
 // 1/sqrt(x) for x in [1, 2]: the hardware estimate refined by one Newton step
 // r <- r + r (1 - x r^2) / 2, so that cs^2 + sn^2 = cs^2 (1 + t^2) is 1 to the
 // FP32 rounding. An estimate left unrefined makes every rotation a rotation
@@ -1014,10 +1003,6 @@ __device__ __forceinline__ void rotation_params_fast(float a, float b, float g, 
   cs = rot_rsqrt(fmaf(t, t, 1.f));
   sn = cs * t;
 }
-__device__ __forceinline__ void rotation_params_fast(double a, double b, double g, double& cs, double& sn) {
-  rotation_params(a, b, g, cs, sn);
-}
-
 // A column pair with each lane's RPL entries held in registers (rows <= 32 RPL):
 // one round of independent loads, the three dot products over the first q rows,
 // and the rotated values stored without reloading.
@@ -1243,9 +1228,13 @@ cudaError_t jacobi_svd(int q, int p, S* W, S* U, S* Sv, S* V, S* Vwork, int max_
   // would keep rotating on noise
   const double eps = (sizeof(C) == 8) ? DBL_EPSILON : (double)FLT_EPSILON;
   const double tol = 4.0 * eps * sqrt((double)q);
+  if constexpr (std::is_same<C, double>::value && std::is_same<S, double>::value) {
+    const cudaError_t e = jacobi_svd64(q, p, W, U, Sv, V, max_sweeps, errw, st);
+    if (e != cudaErrorNotSupported) return e;  // otherwise the one-CTA kernel below
+  }
   // the cluster kernel spreads the columns over JC SMs when there are enough of them (16, an
   // opt-in cluster size, when a block of columns of 8 CTAs does not fit in shared memory)
-  if constexpr (std::is_same<C, S>::value) {
+  if constexpr (std::is_same<C, float>::value && std::is_same<S, float>::value) {
     for (const int nc : {JC, 2 * JC}) {
       const size_t csm = jacobi_cluster_smem<C>(q, p, V != nullptr, nc);
       const int bc = (p + 2 * nc - 1) / (2 * nc), B = bc + (bc & 1);

@@ -1,0 +1,32 @@
+"""tt_svd_truncated at the edges of its kernels' size ranges: the FP64 cluster Jacobi with 1, 8 and 16
+CTAs (changes at 24 and 96 columns; odd and even blocks; plain rotations up to 300 rows of columns and
+accumulated rotations together, scaled ones above)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2606_23274_gb300 import ttfit  # noqa: E402
+
+EPS = np.finfo(np.float64).eps
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (2, 2), (3, 2), (23, 23), (24, 24), (25, 31), (300, 7), (95, 95), (96, 97),
+                                 (129, 127), (1, 600), (900, 24), (200, 120), (281, 33)])
+@pytest.mark.parametrize("floor", [1e-1, 1e-13])
+def test_svd_at_the_edges_of_the_kernels(m, n, floor):
+    rng = np.random.default_rng(m * 2000 + n)
+    r = min(m, n)
+    s = floor ** (np.arange(r) / max(1, r - 1))
+    M = (rng.standard_normal((m, r)) * s) @ rng.standard_normal((r, n))
+    U, S, Vt, _ = ttfit.tt_svd_truncated(M, chi_max=r, tau_rel=0.0)
+    U, S, Vt = U.cpu().numpy(), S.cpu().numpy(), Vt.cpu().numpy()
+    # each of at most 60 sweeps rotates a column r - 1 times, with a rounding of eps each
+    tol = 60 * r * EPS
+    norm = np.linalg.norm(M)
+    assert np.linalg.norm(U * S[None, :] @ Vt - M) <= tol * norm
+    assert np.abs(U.T @ U - np.eye(r)).max() <= tol and np.abs(Vt @ Vt.T - np.eye(r)).max() <= tol
+    assert np.abs(S - np.linalg.svd(M, compute_uv=False)).max() <= tol * norm
