@@ -65,6 +65,11 @@ cudaError_t qr_householder(int q, int p, S* X, S* Q, S* R, cudaStream_t st);
 // cluster kernel does not take run in FP64.
 cudaError_t qr_householder_df32(int q, int p, double* X, double* Q, double* R, cudaStream_t st);
 
+// The same with the columns in registers (qr_reg.cu), which the two above take where it fits (Q may be
+// null); cudaErrorNotSupported otherwise.
+cudaError_t qr_reg64(int q, int p, double* X, double* Q, double* R, cudaStream_t st);
+cudaError_t qr_reg_df32(int q, int p, double* X, double* Q, double* R, cudaStream_t st);
+
 // One-sided Jacobi SVD of the q x p column-major W (q >= p, ld q; overwritten):
 // W = U diag(S) V^T with U (q x p, col-major), S sorted descending, V (p x p,
 // col-major). C is the arithmetic type of the rotations, S the storage type;

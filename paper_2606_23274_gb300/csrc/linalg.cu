@@ -9,6 +9,7 @@
 #include <type_traits>
 #include "common.cuh"
 #include "kernels.h"
+#include "scalar_ops.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -282,56 +283,6 @@ __global__ void __cluster_dims__(JQ, 1, 1) __launch_bounds__(256)
 // gives v = 0, which leaves everything unchanged. Two cluster barriers per
 // panel in the factorisation, one in the formation of Q.
 constexpr int QB = 16;
-
-// Element helpers of the blocked QR for float, double and df32 arithmetic.
-// The df32 square root and reciprocal start from the FP32 result of the high
-// word and take one Newton step in df32 arithmetic, which doubles the number
-// of correct bits (Dekker, Numer. Math. 18 (1971); Karp and Markstein, ACM
-// TOMS 23 (1997)): sqrt(x) = s + (x - s^2) / (2 s), 1/x = r + r (1 - x r).
-__device__ __forceinline__ float qsqrt(float x) { return sqrtf(x); }
-__device__ __forceinline__ double qsqrt(double x) { return sqrt(x); }
-__device__ __forceinline__ df32 qsqrt(df32 x) {
-  if (!(x.hi > 0.0f)) return df32(0.0f, 0.0f);
-  const float s = sqrtf(x.hi);
-  const df32 e = madd(df32(-s, 0.0f), df32(s, 0.0f), x);  // x - s^2
-  return two_sum(s, e.hi * (0.5f / s));
-}
-// 1/sqrt(x): FP32 from the hardware estimate and one Newton step (r (3 - x r^2) / 2)
-__device__ __forceinline__ float qrsqrt(float x) {
-  const float r = rsqrtf(x);
-  return r * fmaf(-0.5f * x * r, r, 1.5f);
-}
-__device__ __forceinline__ double qrsqrt(double x) { return 1.0 / sqrt(x); }
-__device__ __forceinline__ float qrcp(float x) { return 1.0f / x; }
-__device__ __forceinline__ double qrcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ df32 qrcp(df32 x) {
-  const df32 r(1.0f / x.hi, 0.0f);
-  const df32 e = madd(-x, r, df32(1.0f, 0.0f));  // 1 - x r
-  return madd(r, e, r);
-}
-__device__ __forceinline__ df32 qrsqrt(df32 x) { return qrcp(qsqrt(x)); }
-__device__ __forceinline__ bool qneg(float x) { return x < 0.0f; }
-__device__ __forceinline__ bool qneg(double x) { return x < 0.0; }
-__device__ __forceinline__ bool qneg(df32 x) { return x.hi < 0.0f; }  // a normalised pair has the sign of hi
-__device__ __forceinline__ bool qpos(float x) { return x > 0.0f; }
-__device__ __forceinline__ bool qpos(double x) { return x > 0.0; }
-__device__ __forceinline__ bool qpos(df32 x) { return x.hi > 0.0f; }
-template <typename C>
-__device__ __forceinline__ C qshfl_xor(C v, int m) {
-  return __shfl_xor_sync(0xffffffffu, v, m);
-}
-template <>
-__device__ __forceinline__ df32 qshfl_xor<df32>(df32 v, int m) {
-  return df32(__shfl_xor_sync(0xffffffffu, v.hi, m), __shfl_xor_sync(0xffffffffu, v.lo, m));
-}
-template <typename C>
-__device__ __forceinline__ C qshfl(C v, int src) {
-  return __shfl_sync(0xffffffffu, v, src);
-}
-template <>
-__device__ __forceinline__ df32 qshfl<df32>(df32 v, int src) {
-  return df32(__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src));
-}
 
 template <typename C>
 __device__ __forceinline__ void ld16(const C* __restrict__ src, C (&v)[QB]) {
@@ -722,6 +673,10 @@ template <typename C, typename S>
 cudaError_t qr_householder(int q, int p, S* X, S* Q, S* R, cudaStream_t st) {
   if (q <= 0 || p <= 0) return cudaSuccess;
   if (min(q, p) > 1024 || q > 1024) return cudaErrorInvalidValue;
+  if constexpr (std::is_same<C, double>::value && std::is_same<S, double>::value) {
+    const cudaError_t e = qr_reg64(q, p, X, Q, R, st);
+    if (e != cudaErrorNotSupported) return e;
+  }
   if constexpr (std::is_same<C, S>::value) {  // rows spread over a cluster when the matrix is large enough
     const size_t bsm = qr_cluster_blocked_smem<C>(q, p);
     if (Q == nullptr && !(q >= 128 && p >= 16 && bsm <= 220 * 1024)) return cudaErrorInvalidValue;
@@ -764,6 +719,8 @@ cudaError_t qr_householder_df32(int q, int p, double* X, double* Q, double* R, c
   if (q <= 0 || p <= 0) return cudaSuccess;
   const size_t bsm = qr_cluster_blocked_smem<df32>(q, p);
   if (q < 128 || p < 16 || q > 1024 || bsm > 220 * 1024) return qr_householder<double, double>(q, p, X, Q, R, st);
+  const cudaError_t er = qr_reg_df32(q, p, X, Q, R, st);
+  if (er != cudaErrorNotSupported) return er;
   auto launch = [&](auto kern) {
     cudaError_t e = ensure_smem((const void*)kern, bsm);
     if (e != cudaSuccess) return e;

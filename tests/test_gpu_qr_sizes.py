@@ -1,0 +1,42 @@
+"""The Householder QR of the input preparation at the edges of its kernels' size ranges, through
+tt_mpo_compress of chains that lose nothing: every site is factorised as a (bond d d') x bond matrix.
+FP64 arithmetic (precision fp64) and double-FP32 (precision df32)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2606_23274_gb300 import ttfit  # noqa: E402
+
+
+def _dense(cores):
+    T = np.ones((1, 1))
+    for c in cores:
+        T = (T @ c.reshape(c.shape[0], -1)).reshape(-1, c.shape[3])
+    return T.reshape(-1)
+
+
+# legs and bonds; the QR shapes that are the point of each: 1 x 2 .. 2 x 1; 64 x 64, 256 x 128, 512 x 64;
+# 512 x 128; 44 x 33, 132 x 90, 360 x 63 (ragged); 81 x 81, 729 x 113; 208 x 64, 1024 x 29
+@pytest.mark.parametrize("d,bonds", [((1, 2), (1, 2, 1, 2, 1)), ((2, 2), (1, 4, 16, 64, 128, 64, 16, 4, 1)),
+                                     ((2, 2), (1, 4, 16, 64, 128, 128, 64, 16, 4, 1)),
+                                     ((2, 2), (1, 3, 11, 33, 90, 63, 16, 4, 1)), ((3, 3), (1, 9, 81, 113, 81, 9, 1)),
+                                     ((4, 4), (1, 13, 64, 29, 13, 1))])
+@pytest.mark.parametrize("precision,eps", [("fp64", 2.0 ** -52), ("df32", 2.0 ** -44)])
+@pytest.mark.parametrize("null", [False, True])
+def test_preparation_qr_at_the_edges_of_the_kernels(d, bonds, precision, eps, null):
+    rng = np.random.default_rng(sum(bonds))
+    L = len(bonds) - 1
+    X = [rng.standard_normal((bonds[l], *d, bonds[l + 1])) / bonds[l] ** 0.5 for l in range(L)]
+    if null:
+        for l in range(1, L - 1):       # a null column and a multiple of another
+            if bonds[l + 1] > 2:
+                X[l][:, :, :, 1] = 0.0
+                X[l][:, :, :, 2] = X[l][:, :, :, 0] * 2.0
+    C = ttfit.tt_mpo_compress([torch.from_numpy(x).cuda() for x in X], max(bonds), 0.0, precision=precision)
+    got, want = _dense([c.cpu().numpy() for c in C]), _dense(X)
+    # each site: at most 60 sweeps of r rotations, or r reflections, of eps each; twice (preparation, compression)
+    assert np.linalg.norm(got - want) <= 2 * L * 60 * max(bonds) * eps * np.linalg.norm(want)
