@@ -920,7 +920,13 @@ int factorize_body(tt_fit* h, int m, int n, int sweep, int site1, int need) {
       CK(fix_signs<F>(m, n, ks, fUM, m, (F*)nullptr, n, W(h).st));
       return ks;
     }
-    jac(ks, ks, fR2, fU, fS, fV);                 // R2 = Ur S Vr^T
+    if constexpr (std::is_same<F, double>::value) {
+      // on R2^T, whose columns are graded (see svd_tall64): R2^T = Vr S Ur^T
+      copymap<F, F>(h, ks, ks, fR2, IdxMap::lin(1), IdxMap::lin(ks), fX, IdxMap::lin(ks), IdxMap::lin(1));
+      jac(ks, ks, fX, fV, fS, fU);
+    } else {
+      jac(ks, ks, fR2, fU, fS, fV);               // R2 = Ur S Vr^T
+    }
     GemmArgs<F> g3;  // U_M = Q Vr (m x ks)
     g3.M = m; g3.N = ks; g3.K = ks;
     g3.A = fQ; g3.am = IdxMap::lin(1); g3.ak = IdxMap::lin(m); g3.a_kfast = false;
@@ -948,7 +954,9 @@ int factorize_body(tt_fit* h, int m, int n, int sweep, int site1, int need) {
   if (tr) CK(cudaMemcpyAsync(fX, MF, sizeof(F) * (size_t)m * n, cudaMemcpyDeviceToDevice, W(h).st));
   else copymap<F, F>(h, m, n, MF, IdxMap::lin(n), IdxMap::lin(1), fX, IdxMap::lin(1), IdxMap::lin(m));
   F* Ufull;
-  if (q > p) {
+  if constexpr (std::is_same<F, double>::value) {
+    CK(svd_tall64(q, p, fX, fQ, fVw, &Ufull, fS, fV, 60, W(h).errw, h->sm_count, W(h).st));
+  } else if (q > p) {
     qrf(q, p, fX, fQ, fR);                        // X = Qx Rx
     jac(p, p, fR, fU, fS, fV);                    // Rx = Ur S Vr^T
     GemmArgs<F> g;  // Ufull = Qx Ur (q x p)
@@ -2170,15 +2178,27 @@ void zipup_rl(tt_fit* h, const ZipArgs& z, std::vector<double*>& C, std::vector<
       }
       continue;
     }
+    // SVD of Zc (q x p column-major): the left factor's place (T1 or Zc), right factor in V
+    auto zsvd = [&](int q, int pc, T* T1, T* V) -> T* {
+      if constexpr (std::is_same<T, double>::value) {
+        T* U = nullptr;
+        CK(svd_tall64(q, pc, Zc, T1, Vw, &U, Sv, V, 60, w.errw, h->sm_count, st));
+        return U;
+      } else {
+        CK(jacobi_svd<T, T>(q, pc, Zc, T1, Sv, V, Vw, 60, w.errw, st));
+        return T1;
+      }
+    };
     int pv = p;        // singular values in Sv, V = Vn (n x pv column-major)
     T* W_ = nullptr;   // V = Q W when randomized
     if (!rs && m < n) {  // M^T (n x m, column-major = M row-major) is the tall side: M^T = Ux S Vx^T
       CK(cudaMemcpyAsync(Zc, Mr, sizeof(T) * m * n, cudaMemcpyDeviceToDevice, st));
-      CK(jacobi_svd<T, T>((int)n, (int)m, Zc, Vn, Sv, Vx, Vw, 60, w.errw, st));
+      T* U = zsvd((int)n, (int)m, Vn, Vx);
+      if (U != Vn) CK(cudaMemcpyAsync(Vn, U, sizeof(T) * m * n, cudaMemcpyDeviceToDevice, st));
       pv = (int)m;
     } else if (m <= 1024) {  // Z = Ux S W^T
       CK(cudaMemcpyAsync(Zc, Zp, sizeof(T) * m * p, cudaMemcpyDeviceToDevice, st));
-      CK(jacobi_svd<T, T>((int)m, p, Zc, Ux, Sv, rs ? Vx : Vn, Vw, 60, w.errw, st));
+      zsvd((int)m, p, Ux, rs ? Vx : Vn);
       W_ = rs ? Vx : nullptr;
     } else {  // Gram matrix Z^T Z = W S^2 W^T
       GemmArgs<T> g;
@@ -2195,7 +2215,7 @@ void zipup_rl(tt_fit* h, const ZipArgs& z, std::vector<double*>& C, std::vector<
       g.cm = IdxMap::lin(1);
       g.cn = IdxMap::lin(p);
       zgemm<T>(h, g, ws, wse, tc);
-      CK(jacobi_svd<T, T>(p, p, Zc, Ux, Sv, rs ? Vx : Vn, Vw, 60, w.errw, st));
+      zsvd(p, p, Ux, rs ? Vx : Vn);
       CK(sqrt_clamp<T>(p, Sv, st));
       W_ = rs ? Vx : nullptr;
     }

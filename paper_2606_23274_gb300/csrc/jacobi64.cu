@@ -312,10 +312,19 @@ inline size_t jacobi64_smem(int q, int p, bool want_v, int nc) {
 // memory, a smaller one where 16 CTAs cannot be placed. Lanes per pair: 16 in one CTA (8 to 11 pairs,
 // one or two warps on each quadrant), 32 in a cluster, whose CTAs hold few pairs. The scaled rotations
 // pay from 300 rows on (256 x 74: 5.3 ms against 5.6 ms; 128 x 128: 8.2 against 7.9).
-cudaError_t jacobi_svd64(int q, int p, const double* W, double* U, double* Sv, double* V, int max_sweeps,
-                         uint32_t* errw, cudaStream_t st) {
-  const bool want_v = V != nullptr;
-  const double tol = 4.0 * DBL_EPSILON * sqrt((double)q);  // as in jacobi_svd
+namespace {
+
+using Jacobi64Kernel = void (*)(int, int, int, const double*, int, double, uint32_t*, double*, double*, double*);
+
+struct Jacobi64Plan {
+  Jacobi64Kernel kern = nullptr;  // null: does not fit
+  int nc = 0, b = 0;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+};
+
+// The kernel and its launch for a q x p decomposition (plan.cfg points into plan: not to be copied).
+cudaError_t jacobi64_plan(int q, int p, bool want_v, cudaStream_t st, Jacobi64Plan& plan) {
   const bool scaled = q + (want_v ? p : 0) > 300;
   const int order[3][3] = {{1, 8, 16}, {8, 16, 0}, {16, 8, 0}};
   for (const int nc : order[p < 24 ? 0 : p < 96 ? 1 : 2]) {
@@ -325,40 +334,74 @@ cudaError_t jacobi_svd64(int q, int p, const double* W, double* U, double* Sv, d
     const int lp = nc == 1 ? 16 : 32;
     const int threads = std::max(128, 32 * ((B * lp + 31) / 32));
     if (sm > 220 * 1024 || threads > 1024) continue;
-    auto launch = [&](auto kern) -> cudaError_t {
-      cudaError_t e = ensure_smem((const void*)kern, sm);
-      if (e != cudaSuccess) return e;
-      if (nc > 8 && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
-        return e;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(nc);
-      cfg.blockDim = dim3(threads);
-      cfg.dynamicSmemBytes = sm;
-      cfg.stream = st;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = nc;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      if (nc > 8) {  // a 16-CTA cluster must fit in one GPC: check it can be placed
-        int nclu = 0;
-        if (cudaOccupancyMaxActiveClusters(&nclu, kern, &cfg) != cudaSuccess || nclu < 1) {
-          cudaGetLastError();
-          return cudaErrorNotSupported;
-        }
+    Jacobi64Kernel kern = nc == 1 ? (scaled ? jacobi64_kernel<16, true> : jacobi64_kernel<16, false>)
+                                  : (scaled ? jacobi64_kernel<32, true> : jacobi64_kernel<32, false>);
+    cudaError_t e = ensure_smem((const void*)kern, sm);
+    if (e != cudaSuccess) return e;
+    if (nc > 8 && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+      return e;
+    plan.cfg.gridDim = dim3(nc);
+    plan.cfg.blockDim = dim3(threads);
+    plan.cfg.dynamicSmemBytes = sm;
+    plan.cfg.stream = st;
+    plan.at[0].id = cudaLaunchAttributeClusterDimension;
+    plan.at[0].val.clusterDim.x = nc;
+    plan.at[0].val.clusterDim.y = 1;
+    plan.at[0].val.clusterDim.z = 1;
+    plan.cfg.attrs = plan.at;
+    plan.cfg.numAttrs = 1;
+    if (nc > 8) {  // a 16-CTA cluster must fit in one GPC: check it can be placed
+      int nclu = 0;
+      if (cudaOccupancyMaxActiveClusters(&nclu, kern, &plan.cfg) != cudaSuccess || nclu < 1) {
+        cudaGetLastError();
+        continue;
       }
-      ++tl_launches;
-      e = cudaLaunchKernelEx(&cfg, kern, q, p, b, W, max_sweeps, tol, errw, U, Sv, V);
-      return e != cudaSuccess ? e : cudaGetLastError();
-    };
-    cudaError_t e;
-    if (nc == 1) e = scaled ? launch(jacobi64_kernel<16, true>) : launch(jacobi64_kernel<16, false>);
-    else e = scaled ? launch(jacobi64_kernel<32, true>) : launch(jacobi64_kernel<32, false>);
-    if (e != cudaErrorNotSupported) return e;
+    }
+    plan.kern = kern;
+    plan.nc = nc;
+    plan.b = b;
+    return cudaSuccess;
   }
-  return cudaErrorNotSupported;
+  return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t jacobi_svd64(int q, int p, const double* W, double* U, double* Sv, double* V, int max_sweeps,
+                         uint32_t* errw, cudaStream_t st) {
+  const double tol = 4.0 * DBL_EPSILON * sqrt((double)q);  // as in jacobi_svd
+  Jacobi64Plan plan;
+  cudaError_t e = jacobi64_plan(q, p, V != nullptr, st, plan);
+  if (e != cudaSuccess) return e;
+  if (!plan.kern) return cudaErrorNotSupported;
+  ++tl_launches;
+  e = cudaLaunchKernelEx(&plan.cfg, plan.kern, q, p, plan.b, W, max_sweeps, tol, errw, U, Sv, V);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// The same decomposition by way of X = Q R: Jacobi on R^T, whose columns come graded (row i of R is of the
+// size of the i-th singular value), R^T = U' S W^T, so that X = (Q W) S U'^T. On the square or tall matrix
+// itself the columns are of one size and Jacobi needs two to four times the sweeps (128 x 128, spectrum
+// 1 .. 1e-4: 22 against 9; 1 .. 1e-14: 36 against 10). Below 32 columns the QR costs what it saves.
+cudaError_t svd_tall64(int q, int p, double* X, double* T1, double* T2, double** U, double* Sv, double* V,
+                       int max_sweeps, uint32_t* errw, int sm_count, cudaStream_t st) {
+  *U = T1;
+  if (q <= 0 || p <= 0) return cudaSuccess;
+  Jacobi64Plan plan;
+  cudaError_t e = cudaSuccess;
+  if (p >= 32 && q <= 1024 && (e = jacobi64_plan(p, p, true, st, plan)) != cudaSuccess) return e;
+  if (!plan.kern) return jacobi_svd<double, double>(q, p, X, T1, Sv, V, T2, max_sweeps, errw, st);
+  e = qr_householder<double, double>(q, p, X, T1, T2, st);  // Q: T1, R: T2
+  if (e != cudaSuccess) return e;
+  const IdxMap one = IdxMap::lin(1), row = IdxMap::lin(p);
+  if ((e = copy_map<double, double>(p, p, T2, one, row, X, row, one, 1.0, st)) != cudaSuccess) return e;
+  if ((e = jacobi_svd64(p, p, X, V, Sv, T2, max_sweeps, errw, st)) != cudaSuccess) return e;
+  GemmArgs<double> g;  // U = Q W
+  g.M = q; g.N = p; g.K = p;
+  g.A = T1; g.am = one; g.ak = IdxMap::lin(q); g.a_kfast = false;
+  g.B = T2; g.bn = row; g.bk = one;
+  g.C = *U = X; g.cm = one; g.cn = IdxMap::lin(q);
+  return gemm_simt<double>(g, nullptr, 0, sm_count, st);
 }
 
 }  // namespace ttfit

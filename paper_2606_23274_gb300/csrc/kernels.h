@@ -84,6 +84,11 @@ cudaError_t jacobi_svd(int q, int p, S* W, S* U, S* Sv, S* V, S* Vwork, int max_
 cudaError_t jacobi_svd64(int q, int p, const double* W, double* U, double* Sv, double* V, int max_sweeps,
                          uint32_t* errw, cudaStream_t st);
 
+// SVD of the q x p column-major X (q >= p; overwritten) as jacobi_svd<double> gives it, by way of a QR
+// where that saves sweeps. T1 (q x p), T2 (p x p): scratch. *U: where the left factor is, X or T1.
+cudaError_t svd_tall64(int q, int p, double* X, double* T1, double* T2, double** U, double* Sv, double* V,
+                       int max_sweeps, uint32_t* errw, int sm_count, cudaStream_t st);
+
 // ||X||_F of n values (type T) into *out (double), flags non-finite values.
 template <typename T>
 cudaError_t frob_norm(const T* x, long long n, double* out, uint32_t* errw, cudaStream_t st);

@@ -63,7 +63,10 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   else e = copy_map<double, double>(m, n, M, IdxMap::lin(n), IdxMap::lin(1), X, IdxMap::lin(1), IdxMap::lin(m), 1.0, st);
   if (e != cudaSuccess) return e;
   if ((e = frob_norm<double>(M, (long long)m * n, nrm, info, st)) != cudaSuccess) return e;
-  if ((e = jacobi_svd<double, double>(q, r, X, Ux, Sv, Vx, Vw, 60, info, st)) != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = svd_tall64(q, r, X, Ux, Vw, &Ux, Sv, Vx, 60, info, sms, st)) != cudaSuccess) return e;
   if ((e = fix_signs<double>(tr ? r : q, tr ? q : r, r, tr ? Vx : Ux, tr ? r : q, tr ? Ux : Vx, tr ? q : r, st)) !=
       cudaSuccess)
     return e;
