@@ -1263,87 +1263,120 @@ template cudaError_t jacobi_svd<float, float>(int, int, float*, float*, float*, 
                                               cudaStream_t);
 
 // ---------------------------------------------------------------------------
+// ||x||: one cluster of up to 8 CTAs, partial sums joined in the first one's shared memory (one CTA alone
+// is bound by its SM: 262144 FP64 values take it 100 us, eight 15 us). Up to 8192 values one CTA.
+template <typename T>
+__device__ __forceinline__ void norm_add(T v, T& part) { part += v * v; }
+// double-FP32 values: the norm is taken of hi + lo in FP64
+__device__ __forceinline__ void norm_add(df32 x, double& part) {
+  const double v = (double)x;
+  part += v * v;
+}
 template <typename T>
 __global__ void __launch_bounds__(1024) frob_kernel(const T* __restrict__ x, long long n, double* out, uint32_t* errw) {
+  // per-thread partial in the value type (FP32 stays on the FP32 pipes)
+  using P = typename std::conditional<std::is_same<T, float>::value, float, double>::type;
+  cg::cluster_group cl = cg::this_cluster();
   __shared__ double red[32];
-  T part = 0;  // per-thread partial in the value type (FP32 stays on the FP32 pipes)
+  __shared__ double total[8];
+  P part = 0;
   bool bad = false;
-  for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+#pragma unroll 4
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const T v = x[i];
-    bad |= !isfinite(v);
-    part += v * v;
+    if constexpr (std::is_same<T, df32>::value) bad |= !isfinite(v.hi + v.lo);
+    else bad |= !isfinite(v);
+    norm_add(v, part);
   }
-  double s = block_sum((double)part, red);
+  const double s = block_sum((double)part, red);
   bad = __syncthreads_or(bad);
   if (threadIdx.x == 0) {
-    *out = sqrt(s);
+    *cl.map_shared_rank(&total[blockIdx.x], 0) = s;
     if (bad && errw) atomicOr(errw, ERRW_NAN);
   }
-}
-
-// double-FP32 values: the norm is taken of hi + lo in FP64 (small arrays only)
-template <>
-__global__ void __launch_bounds__(1024) frob_kernel<df32>(const df32* __restrict__ x, long long n, double* out,
-                                                           uint32_t* errw) {
-  __shared__ double red[32];
-  double part = 0;
-  bool bad = false;
-  for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-    const double v = (double)x[i];
-    bad |= !isfinite(v);
-    part += v * v;
-  }
-  double s = block_sum(part, red);
-  bad = __syncthreads_or(bad);
-  if (threadIdx.x == 0) {
-    *out = sqrt(s);
-    if (bad && errw) atomicOr(errw, ERRW_NAN);
+  cl.sync();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double t = 0;
+    for (unsigned c = 0; c < gridDim.x; ++c) t += total[c];
+    *out = sqrt(t);
   }
 }
 
 template <typename T>
 cudaError_t frob_norm(const T* x, long long n, double* out, uint32_t* errw, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n <= 8192 ? 1 : 8);  // one cluster
+  cfg.blockDim = dim3(1024);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cfg.gridDim.x;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   ++tl_launches;
-  frob_kernel<T><<<1, 1024, 0, st>>>(x, n, out, errw);
-  return cudaGetLastError();
+  cudaError_t e = cudaLaunchKernelEx(&cfg, frob_kernel<T>, x, n, out, errw);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 template cudaError_t frob_norm<double>(const double*, long long, double*, uint32_t*, cudaStream_t);
 template cudaError_t frob_norm<float>(const float*, long long, double*, uint32_t*, cudaStream_t);
 template cudaError_t frob_norm<df32>(const df32*, long long, double*, uint32_t*, cudaStream_t);
 
 // ---------------------------------------------------------------------------
+// One warp; lane i holds the i-th run of consecutive values, the tails come from a suffix scan over the
+// runs (one thread's chain of FP64 operations took 51 us for 256 values, this takes 7).
+__device__ __forceinline__ double suffix_from(double v, int lane) {  // sum over the lanes >= lane
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double u = __shfl_down_sync(0xffffffffu, v, o);
+    if (lane + o < 32) v += u;
+  }
+  return v;
+}
 template <typename F>
 __global__ void truncate_kernel(const F* S, int p, const double* normM, double tau_over_L, int chi_max,
                                 double cutoff, int* info, double* dinfo) {
-  if (threadIdx.x != 0) return;
+  const int lane = threadIdx.x;
+  const int run = (p + 31) / 32, j0 = min(p, lane * run), j1 = min(p, j0 + run);
   const double nM = *normM;
+  double sq = 0.0;  // of my run
+  for (int j = j1 - 1; j >= j0; --j) sq += (double)S[j] * (double)S[j];
   int k = min(chi_max, p);
   if (tau_over_L > 0.0) {
+    // the smallest j >= 1 whose tail (sum over i >= j of s_i^2) is within the threshold; tails grow as j falls
     const double thr = tau_over_L * nM;
+    double tail = __shfl_down_sync(0xffffffffu, suffix_from(sq, lane), 1);
+    if (lane == 31) tail = 0.0;
     int kmin = p;
-    double tail = 0.0;
-    for (int j = p - 1; j >= 1; --j) {
+    for (int j = j1 - 1; j >= max(j0, 1); --j) {
       tail += (double)S[j] * (double)S[j];
       if (sqrt(tail) <= thr) kmin = j;
       else break;
     }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
     k = min(k, kmin);
   }
   if (p > 0) {
     int cnt = 0;
-    for (int j = 0; j < p; ++j) cnt += (double)S[j] > cutoff * (double)S[0];
-    k = min(k, cnt);
+    const double lim = cutoff * (double)S[0];
+    for (int j = j0; j < j1; ++j) cnt += (double)S[j] > lim;
+    k = min(k, __reduce_add_sync(0xffffffffu, cnt));
   }
   k = max(k, 1);
   double kept = 0.0, disc = 0.0;
-  for (int j = 0; j < p; ++j) {
+  for (int j = j0; j < j1; ++j) {
     const double sj = (double)S[j];
     if (j < k) kept += sj * sj;
     else disc += sj * sj;
   }
-  info[0] = k;
-  dinfo[0] = kept;
-  dinfo[1] = nM > 0.0 ? sqrt(disc) / nM : 0.0;
+  kept = warp_sum(kept);
+  disc = warp_sum(disc);
+  if (lane == 0) {
+    info[0] = k;
+    dinfo[0] = kept;
+    dinfo[1] = nM > 0.0 ? sqrt(disc) / nM : 0.0;
+  }
 }
 
 template <typename F>
