@@ -474,16 +474,23 @@ __global__ void oz_slice_kernel(int R, int K, int Kp, const T* __restrict__ X, l
   if (e == INT_MIN) e = OZ_EZERO;
   if (lane == 0) ex[(long long)row * nch + ch] = e;
   const size_t plane = (size_t)R * Kp;
+  // 7 - e = q1 + q2, both factors normal (e is -126 .. 129, or OZ_EZERO where every x is zero)
+  const int q1 = e == OZ_EZERO ? 0 : (7 - e) / 2, q2 = e == OZ_EZERO ? 0 : 7 - e - q1;
+  const float s1 = __int_as_float((q1 + 127) << 23), s2 = __int_as_float((q2 + 127) << 23);
+#pragma unroll 2
   for (int k = k0 + lane; k < kp1; k += 32) {
     float d[OZ_S];
     if (k < K) {
       const float2 v = as_pair<T>(x[k]);
-      // x 2^(7-e) = th + tl exactly; peel one 8-bit digit per level, carrying the exact remainder
-      float th = scalbnf(v.x, 7 - e), tl = scalbnf(v.y, 7 - e);
+      // x 2^(7-e) = th + tl exactly; peel one 8-bit digit per level, carrying the exact remainder.
+      // Powers of two are multiplied (s1 s2 = 2^(7-e)): exact as scalbnf is, without its range checks
+      float th = v.x * s1 * s2, tl = v.y * s1 * s2;
+      float w = 1.f;
 #pragma unroll
       for (int i = 0; i < OZ_S; ++i) {
         const float si = rintf(th);
-        d[i] = scalbnf(si, -8 * i);
+        d[i] = si * w;
+        w *= 0x1p-8f;
         const df32 r = two_sum(__fsub_rn(th, si), tl);  // th - si is exact
         th = __fmul_rn(r.hi, 256.f);
         tl = __fmul_rn(r.lo, 256.f);

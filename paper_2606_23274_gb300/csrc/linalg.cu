@@ -1456,26 +1456,96 @@ template cudaError_t gauge_update<df32, double>(int, int, int, const double*, in
                                                 const int*, double*, double*, double*, df32*, df32*, cudaStream_t);
 
 // ---------------------------------------------------------------------------
-template <typename Tin, typename Tout>
+// SCALED is a template parameter, not a test of `scale` in the kernel: the compiler evaluates both sides of
+// such a test, and the conversions and the product keep an SM's FP64 pipe busy for 60 cycles a warp
+// (a plain FP32 copy of 85 MB took 167 us so). Offsets fit 32-bit divisions below 2^31 elements.
+template <typename Tin, typename Tout, bool SCALED>
 __global__ void copy_map_kernel(int rows, int cols, const Tin* __restrict__ in, IdxMap im, IdxMap in_,
                                 Tout* __restrict__ out, IdxMap om, IdxMap on, double scale) {
   const long long tot = (long long)rows * cols;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e / cols), j = (int)(e % cols);
+    int i, j;
+    if (rows == 1) {
+      i = 0, j = (int)e;
+    } else if (tot <= 0x7FFFFFFF) {
+      i = (int)((unsigned)e / (unsigned)cols), j = (int)((unsigned)e - (unsigned)i * (unsigned)cols);
+    } else {
+      i = (int)(e / cols), j = (int)(e % cols);
+    }
     const Tin x = in[im(i) + in_(j)];
-    out[om(i) + on(j)] = scale == 1.0 ? (Tout)x : (Tout)(scale * (double)x);  // plain copies stay off the FP64 pipe
+    if constexpr (SCALED) out[om(i) + on(j)] = (Tout)(scale * (double)x);
+    else out[om(i) + on(j)] = (Tout)x;
   }
 }
+
+// A transposing copy: the input runs fastest along the rows, the output along the columns. 32 x 32 tiles go
+// through shared memory, so that both sides move whole lines.
+template <typename Tin, typename Tout, bool SCALED>
+__global__ void __launch_bounds__(256) copy_map_tiled_kernel(int rows, int cols, const Tin* __restrict__ in, IdxMap im,
+                                                             IdxMap in_, Tout* __restrict__ out, IdxMap om, IdxMap on,
+                                                             double scale) {
+  __shared__ Tin tile[32][33];
+  __shared__ long long ir[32], ic[32], orow[32], oc[32];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int nct = (cols + 31) / 32;
+  const long long ntile = (long long)nct * ((rows + 31) / 32);
+  for (long long t = blockIdx.x; t < ntile; t += gridDim.x) {
+    const int i0 = (int)(t / nct) * 32, j0 = (int)(t % nct) * 32;
+    if (ty < 4) {  // offsets of the tile's rows and columns, once
+      const int i = min(i0 + tx, rows - 1), j = min(j0 + tx, cols - 1);
+      if (ty == 0) ir[tx] = im(i);
+      else if (ty == 1) ic[tx] = in_(j);
+      else if (ty == 2) orow[tx] = om(i);
+      else oc[tx] = on(j);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = ty; k < 32; k += 8)  // lanes along the rows: the input's fast direction
+      if (i0 + tx < rows && j0 + k < cols) tile[k][tx] = in[ir[tx] + ic[k]];
+    __syncthreads();
+#pragma unroll
+    for (int k = ty; k < 32; k += 8)
+      if (i0 + k < rows && j0 + tx < cols) {
+        const Tin x = tile[tx][k];
+        if constexpr (SCALED) out[orow[k] + oc[tx]] = (Tout)(scale * (double)x);
+        else out[orow[k] + oc[tx]] = (Tout)x;
+      }
+    __syncthreads();
+  }
+}
+
+// Whether the innermost level of a map steps through neighbouring memory.
+inline bool unit_inner(const IdxMap& m) { return m.s2 == 1; }
 
 template <typename Tin, typename Tout>
 cudaError_t copy_map(int rows, int cols, const Tin* in, IdxMap im, IdxMap in_, Tout* out, IdxMap om, IdxMap on,
                      double scale, cudaStream_t st) {
   long long tot = (long long)rows * cols;
   if (tot <= 0) return cudaSuccess;
-  int blocks = (int)((tot + 255) / 256);
-  if (blocks > 4096) blocks = 4096;
   ++tl_launches;
-  copy_map_kernel<Tin, Tout><<<blocks, 256, 0, st>>>(rows, cols, in, im, in_, out, om, on, scale);
+  // transposing copies from 32 x 32 on; below, and where both sides run along the columns (or neither runs
+  // along one), one thread an element; where both run along the rows (column-major copies), so do the threads
+  const bool rows_in = unit_inner(im) && !unit_inner(in_), cols_out = unit_inner(on) && !unit_inner(om);
+  const bool cols_in = unit_inner(in_) && !unit_inner(im), rows_out = unit_inner(om) && !unit_inner(on);
+  const bool tiled = rows >= 32 && cols >= 32 && ((rows_in && cols_out) || (cols_in && rows_out));
+  if ((tiled && cols_in) || (!tiled && rows_in && rows_out)) {  // swap the roles of rows and columns
+    std::swap(rows, cols);
+    std::swap(im, in_);
+    std::swap(om, on);
+  }
+  auto go = [&](auto scaled) {
+    constexpr bool SC = decltype(scaled)::value;
+    if (tiled) {
+      const long long tiles = (long long)((rows + 31) / 32) * ((cols + 31) / 32);
+      const int blocks = (int)(tiles < (1 << 16) ? tiles : (1 << 16));
+      copy_map_tiled_kernel<Tin, Tout, SC><<<blocks, 256, 0, st>>>(rows, cols, in, im, in_, out, om, on, scale);
+    } else {
+      int blocks = (int)((tot + 255) / 256 < 4096 ? (tot + 255) / 256 : 4096);
+      copy_map_kernel<Tin, Tout, SC><<<blocks, 256, 0, st>>>(rows, cols, in, im, in_, out, om, on, scale);
+    }
+  };
+  if (scale == 1.0) go(std::false_type{});
+  else go(std::true_type{});
   return cudaGetLastError();
 }
 template cudaError_t copy_map<double, double>(int, int, const double*, IdxMap, IdxMap, double*, IdxMap, IdxMap, double,
