@@ -104,6 +104,134 @@ __global__ void __launch_bounds__(NT, 3) gemm_simt_kernel(GemmArgs<T> g, T* __re
   }
 }
 
+// FP32. 128 threads, each 8 x 4 outputs (rows 8 ty .. 8 ty + 7, columns tx + TX j); k-tiles of 16 in two shared
+// buffers, the next one's loads in registers while the present one is multiplied, and the k offsets of 256 terms
+// tabulated at a time. The kernel above waits for its loads and evaluates the k maps in every k-tile: for the
+// gradient's products (3072 x 384 x 96, 6144 x 192 x 192, 9216 x 32 x 128) it was bound by that latency, at
+// 5 TFLOP/s. Sums run in the same order, so the results are the same bits.
+template <int BM, int BN>
+__global__ void __launch_bounds__(128) gemm_f32_kernel(GemmArgs<float> g, float* __restrict__ ws, int k_per_split) {
+  constexpr int TX = BN / 4, KC = 256, NA = BM * BK / 128, NB = BN * BK / 128;
+  static_assert(TX * (BM / 8) == 128, "8 x 4 outputs a thread");
+  __shared__ __align__(16) float As[2][BK][BM + 4];
+  __shared__ float Bs[2][BK][BN + 1];
+  __shared__ long long arow[BM], brow[BN];
+  __shared__ long long akoff[KC], bkoff[KC];
+  const int tid = threadIdx.x;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int kb = blockIdx.z * k_per_split;
+  const int ke = min(g.K, kb + k_per_split);
+  for (int t = tid; t < BM + BN; t += 128) {
+    if (t < BM) arow[t] = (m0 + t < g.M) ? g.am(m0 + t) : 0;
+    else brow[t - BM] = (n0 + t - BM < g.N) ? g.bn(n0 + t - BM) : 0;
+  }
+  const int tx = tid % TX, ty = tid / TX;
+  float acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  float ra[NA], rb[NB];
+  auto load = [&](int k0) {
+    const int c0 = (k0 - kb) % KC;
+    if (c0 == 0) {  // the next stretch of k offsets
+      __syncthreads();
+      for (int t = tid; t < KC; t += 128) {
+        akoff[t] = k0 + t < ke ? g.ak(k0 + t) : 0;
+        bkoff[t] = k0 + t < ke ? g.bk(k0 + t) : 0;
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int e = tid + 128 * i;
+      const int r = g.a_kfast ? e / BK : e % BM, kk = g.a_kfast ? e % BK : e / BM;
+      ra[i] = (m0 + r < g.M && k0 + kk < ke) ? g.A[arow[r] + akoff[c0 + kk]] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int e = tid + 128 * i;
+      const int r = g.b_kfast ? e / BK : e % BN, kk = g.b_kfast ? e % BK : e / BN;
+      rb[i] = (n0 + r < g.N && k0 + kk < ke) ? g.B[brow[r] + bkoff[c0 + kk]] : 0.f;
+    }
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int e = tid + 128 * i;
+      const int r = g.a_kfast ? e / BK : e % BM, kk = g.a_kfast ? e % BK : e / BM;
+      As[buf][kk][r] = ra[i];
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int e = tid + 128 * i;
+      const int r = g.b_kfast ? e / BK : e % BN, kk = g.b_kfast ? e % BK : e / BN;
+      Bs[buf][kk][r] = rb[i];
+    }
+  };
+  if (kb < ke) {
+    load(kb);
+    store(0);
+    __syncthreads();
+    int buf = 0;
+    for (int k0 = kb; k0 < ke; k0 += BK) {
+      const bool more = k0 + BK < ke;
+      if (more) load(k0 + BK);
+#pragma unroll
+      for (int kk = 0; kk < BK; ++kk) {
+        const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][8 * ty]);
+        const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][8 * ty + 4]);
+        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        float b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j] = Bs[buf][kk][tx + TX * j];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      }
+      if (more) store(buf ^ 1);
+      buf ^= 1;
+      __syncthreads();
+    }
+  }
+  if (ws) {  // split-K partial: dense [split][M][N]
+    float* w = ws + (size_t)blockIdx.z * g.M * g.N;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int m = m0 + 8 * ty + i;
+      if (m >= g.M) continue;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int n = n0 + tx + TX * j;
+        if (n < g.N) w[(size_t)m * g.N + n] = acc[i][j];
+      }
+    }
+    return;
+  }
+  long long cn[4], cn2[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int n = min(n0 + tx + TX * j, g.N - 1);
+    cn[j] = g.cn(n);
+    cn2[j] = g.C2 ? g.cn2(n) : 0;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int m = m0 + 8 * ty + i;
+    if (m >= g.M) continue;
+    const long long cr = g.cm(m), cr2 = g.C2 ? g.cm2(m) : 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (n0 + tx + TX * j >= g.N) continue;
+      float v = g.alpha * acc[i][j];
+      if (g.C2) g.C2[cr2 + cn2[j]] = v;
+      if (g.beta != 0.f) v += g.beta * g.C[cr + cn[j]];
+      g.C[cr + cn[j]] = v;
+    }
+  }
+}
+
 // Sum of the split-K partials into the output layouts. A block takes 8 rows of 32 columns: the partials are read
 // along the columns, each output is written along its own fast direction, and the index maps are evaluated once
 // a row and column of the tile (four maps and a 64-bit division an element took 20 us for 512 x 512 df32).
@@ -174,12 +302,15 @@ cudaError_t gemm_simt(const GemmArgs<T>& g, T* ws, size_t ws_elems, int sm_count
   auto tiles_of = [&](int mt) { return (long long)((g.M + 16 * mt - 1) / (16 * mt)) * ((g.N + 16 * mt - 1) / (16 * mt)); };
   // FP64 and df32: the largest of 64, 32 and 16 that gives two tiles an SM. FP64 gradient of chi = 12
   // (products of 288 x 24 x 24 and the like): 39 us a launch with tiles of 64, 10 us so; 1.58 ms
-  // against 4.44 ms for the call. FP32 keeps 64: its tiles are bound by their loads.
+  // against 4.44 ms for the call. FP32 has tiles of its own.
   int mt = 4;
   if (slow)
     while (mt > 1 && tiles_of(mt) < 2 * sm_count) mt /= 2;
-  const int tb = 16 * mt;
-  int gm = (g.M + tb - 1) / tb, gn = (g.N + tb - 1) / tb;
+  int tbm = 16 * mt, tbn = 16 * mt;
+  // FP32: 64 x 64 tiles, 128 x 32 or 32 x 128 where one side is no wider than 32
+  if (!slow && g.N <= 32) tbm = 128, tbn = 32;
+  else if (!slow && g.M <= 32) tbm = 32, tbn = 128;
+  int gm = (g.M + tbm - 1) / tbm, gn = (g.N + tbn - 1) / tbn;
   int tiles = gm * gn;
   int splits = 1;
   // split K while the grid covers fewer than two waves of the SMs and each
@@ -199,7 +330,9 @@ cudaError_t gemm_simt(const GemmArgs<T>& g, T* ws, size_t ws_elems, int sm_count
     else if (mt == 2) gemm_simt_kernel<T, 2><<<grid, NT, 0, st>>>(g, wsp, kps);
     else gemm_simt_kernel<T, 4><<<grid, NT, 0, st>>>(g, wsp, kps);
   } else {
-    gemm_simt_kernel<T, 4><<<grid, NT, 0, st>>>(g, wsp, kps);
+    if (tbn == 32) gemm_f32_kernel<128, 32><<<grid, 128, 0, st>>>(g, wsp, kps);
+    else if (tbm == 32) gemm_f32_kernel<32, 128><<<grid, 128, 0, st>>>(g, wsp, kps);
+    else gemm_f32_kernel<64, 64><<<grid, 128, 0, st>>>(g, wsp, kps);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || splits == 1) return e;
