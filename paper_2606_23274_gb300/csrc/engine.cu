@@ -138,6 +138,29 @@ BlockCache& block_cache() {
   return *c;
 }
 
+}  // namespace
+
+namespace ttfit {
+
+void* block_take(int dev, size_t bytes, size_t* got) {
+  bytes = (std::max<size_t>(bytes, 1) + 511) & ~(size_t)511;
+  *got = bytes;
+  void* p = block_cache().take(dev, bytes, got);
+  if (p) return p;
+  if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+  cudaGetLastError();
+  block_cache().trim(dev);
+  if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+  cudaGetLastError();
+  return nullptr;
+}
+
+void block_give(int dev, size_t bytes, void* p) { block_cache().give(dev, bytes, p); }
+
+}  // namespace ttfit
+
+namespace {
+
 // Device allocations owned by a handle (from the block cache).
 struct DevPool {
   struct Blk {
@@ -150,25 +173,12 @@ struct DevPool {
   template <typename T>
   T* alloc(size_t n) {
     if (fault & TT_FAULT_ALLOC_FAIL) throw TTError(TT_ERR_OUT_OF_MEMORY, "injected allocation failure");
-    if (n == 0) n = 1;
-    const size_t bytes = (n * sizeof(T) + 511) & ~(size_t)511;
     int dev = 0;
     cudaGetDevice(&dev);
-    size_t got = bytes;
-    void* p = block_cache().take(dev, bytes, &got);
-    if (!p) {
-      cudaError_t e = cudaMalloc(&p, bytes);
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        block_cache().trim(dev);
-        e = cudaMalloc(&p, bytes);
-      }
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        throw TTError(TT_ERR_OUT_OF_MEMORY, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
-      }
-    }
-    blks.push_back({p, p ? got : bytes, dev});
+    size_t got = 0;
+    void* p = block_take(dev, n * sizeof(T), &got);
+    if (!p) throw TTError(TT_ERR_OUT_OF_MEMORY, "cudaMalloc of " + std::to_string(got) + " bytes failed");
+    blks.push_back({p, got, dev});
     return (T*)p;
   }
   void release(void* p) {

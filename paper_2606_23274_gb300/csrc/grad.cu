@@ -45,22 +45,32 @@ struct GradError : std::runtime_error {
                       std::string(#__VA_ARGS__) + ": " + cudaGetErrorString(e_));                       \
   } while (0)
 
-// Device buffers owned by one call.
+// Device buffers of one call, from the process-wide block cache (a call takes 60 to 200 of them: cudaMalloc and
+// cudaFree were 0.9 ms of the 1.6 ms of a short FP64 gradient). The stream is synchronised before they go back, also
+// when the call fails.
 struct Arena {
-  std::vector<void*> ptrs;
+  struct Blk {
+    void* p;
+    size_t bytes;
+  };
+  std::vector<Blk> blks;
+  int dev = 0;
+  cudaStream_t st;
+  explicit Arena(cudaStream_t s) : st(s) { cudaGetDevice(&dev); }
   template <typename T>
   T* alloc(size_t n) {
-    void* p = nullptr;
-    if (cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T)) != cudaSuccess) {
-      cudaGetLastError();
-      throw GradError(TT_ERR_OUT_OF_MEMORY, "cudaMalloc of " + std::to_string(n * sizeof(T)) + " bytes failed");
-    }
-    ptrs.push_back(p);
+    size_t got = 0;
+    void* p = block_take(dev, std::max<size_t>(n, 1) * sizeof(T), &got);
+    if (!p) throw GradError(TT_ERR_OUT_OF_MEMORY, "cudaMalloc of " + std::to_string(n * sizeof(T)) + " bytes failed");
+    blks.push_back({p, got});
     return (T*)p;
   }
   ~Arena() {
-    for (void* p : ptrs) cudaFree(p);
+    if (!blks.empty()) cudaStreamSynchronize(st);
+    for (auto& b : blks) block_give(dev, b.bytes, b.p);
   }
+  Arena(const Arena&) = delete;
+  Arena& operator=(const Arena&) = delete;
 };
 
 using Ext = std::map<char, long long>;
@@ -332,7 +342,7 @@ void store_cores(const T* in, const tt_mpo_desc* d, int l, long long n, cudaStre
 template <typename T>
 double run_grad(const tt_mpo_desc* Ad, const tt_mpo_desc* Bd, const tt_mpo_desc* Xd, int target, int ckpt,
                 cudaStream_t st, const tt_mpo_desc* gAd, const tt_mpo_desc* gBd, bool tc = false) {
-  Arena ar;
+  Arena ar(st);
   Grad<T> G(ar);
   int LA, LB, LX, LgA, LgB;
   std::vector<int> doA, diA, bA, doB, diB, bB, doX, diX, bX, o1, i1, b1, o2, i2, b2;

@@ -94,11 +94,14 @@ extern "C" tt_status tt_svd_truncated(const double* M, int m, int n, int chi_max
   if (s != TT_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t nd = svd_scratch_doubles(m, n);
-  double* scratch = nullptr;
-  if (cudaMalloc(&scratch, nd * sizeof(double)) != cudaSuccess) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
-    return TT_ERR_OUT_OF_MEMORY;
+    return TT_ERR_CUDA;
   }
+  size_t got = 0;
+  double* scratch = (double*)block_take(dev, nd * sizeof(double), &got);
+  if (!scratch) return TT_ERR_OUT_OF_MEMORY;
   int* k_dev = (int*)(scratch + nd - 1);
   cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, k_dev, scratch, st);
   int k = 0;
@@ -106,8 +109,9 @@ extern "C" tt_status tt_svd_truncated(const double* M, int m, int n, int chi_max
   if (e == cudaSuccess) e = cudaMemcpyAsync(&k, k_dev, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(flags, scratch + svd_info_offset(m, n), 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(scratch);
+  const cudaError_t es = cudaStreamSynchronize(st);  // before the block goes back, whatever failed
+  if (e == cudaSuccess) e = es;
+  block_give(dev, got, scratch);
   if (e != cudaSuccess) return TT_ERR_CUDA;
   if (flags[0] & (ERRW_NAN | ERRW_NOCONV)) return TT_ERR_NUMERICAL;
   *k_out = k;
