@@ -32,10 +32,11 @@ namespace tc {
 
 constexpr int BM = 128, BN = 128, BK = 32;  // BK fp32 elements = 128 bytes = one swizzle span
 constexpr int TILE_BYTES = BM * BK * 4;     // 16 KB (A); B tile has the same size
-// 1-pass TF32: 4 stages of (A, B); split (3xTF32): 3 stages of (A, B, A_lo, B_lo)
-template <bool SPLIT>
+// 1-pass TF32: 4 stages of (A, B); split (3xTF32): 3 stages of (A, B, A_lo, B_lo), or one (OVERLAP), so that
+// three CTAs share an SM and one's loads, split and epilogue run under the others' products
+template <bool SPLIT, bool OVERLAP = false>
 struct Cfg {
-  static constexpr int STAGES = SPLIT ? 3 : 4;
+  static constexpr int STAGES = OVERLAP ? 1 : SPLIT ? 3 : 4;
   static constexpr int TILES = SPLIT ? 4 : 2;
   static constexpr int SMEM_BYTES = STAGES * TILES * TILE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
 };
@@ -123,12 +124,12 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-template <bool B_MN, bool SPLIT>
-__global__ void __launch_bounds__(128, 1)
+template <bool B_MN, bool SPLIT, bool OVERLAP>
+__global__ void __launch_bounds__(128, OVERLAP ? 3 : 1)
     gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N,
                      int K, int k_per_split, float* __restrict__ C, IdxMap cm, IdxMap cn, float alpha, float beta,
                      float* __restrict__ C2, IdxMap cm2, IdxMap cn2, float* __restrict__ ws, uint32_t* errw) {
-  constexpr int STAGES = Cfg<SPLIT>::STAGES;
+  constexpr int STAGES = Cfg<SPLIT, OVERLAP>::STAGES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = smem;
@@ -657,6 +658,13 @@ __global__ void __launch_bounds__(128, 1)
 
 }  // namespace tc
 
+// Whether gemm_tf32's TMA can load this operand as it lies: K contiguous, base and rows 16-byte aligned.
+bool tf32_loadable(const float* p, const IdxMap& rows, const IdxMap& k, int K) {
+  long long ld, one;
+  return tc::lin_stride(rows, ld) && tc::lin_stride(k, one) && one == 1 && ((uintptr_t)p & 15) == 0 && (ld * 4) % 16 == 0 &&
+         ld >= K;
+}
+
 // Returns cudaErrorNotSupported when the operand layouts cannot be fed by TMA
 // (the caller then uses the CUDA-core kernel).
 cudaError_t gemm_tf32(const GemmArgs<float>& g, float* ws, size_t ws_elems, int sm_count, uint32_t* errw,
@@ -680,9 +688,6 @@ cudaError_t gemm_tf32(const GemmArgs<float>& g, float* ws, size_t ws_elems, int 
   } else {
     if (!make_map(&tb, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)ldb, 32, BK)) return cudaErrorNotSupported;
   }
-  cudaError_t ea = split ? ensure_smem((const void*)gemm_tf32_kernel<false, true>, Cfg<true>::SMEM_BYTES)
-                         : ensure_smem((const void*)gemm_tf32_kernel<false, false>, Cfg<false>::SMEM_BYTES);
-  if (ea != cudaSuccess) return ea;
   const int gm = (g.M + BM - 1) / BM, gn = (g.N + BN - 1) / BN;
   int splits = 1;
   while (gm * gn * splits < sm_count && g.K / (splits * 2) >= 4 * BK && (size_t)(splits * 2) * g.M * g.N <= ws_elems)
@@ -692,14 +697,19 @@ cudaError_t gemm_tf32(const GemmArgs<float>& g, float* ws, size_t ws_elems, int 
   splits = (g.K + kps - 1) / kps;
   dim3 grid(gn, gm, splits);
   float* wsp = splits > 1 ? ws : nullptr;
-  ++tl_launches;
-  if (split)
-    gemm_tf32_kernel<false, true><<<grid, 128, Cfg<true>::SMEM_BYTES, st>>>(
-        ta, tb, g.M, g.N, g.K, kps, g.C, g.cm, g.cn, g.alpha, g.beta, g.C2, g.cm2, g.cn2, wsp, errw);
-  else
-    gemm_tf32_kernel<false, false><<<grid, 128, Cfg<false>::SMEM_BYTES, st>>>(
-        ta, tb, g.M, g.N, g.K, kps, g.C, g.cm, g.cn, g.alpha, g.beta, g.C2, g.cm2, g.cn2, wsp, errw);
-  cudaError_t e = cudaGetLastError();
+  auto launch = [&](auto kern, size_t smem) -> cudaError_t {
+    cudaError_t e = ensure_smem((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    ++tl_launches;
+    kern<<<grid, 128, smem, st>>>(ta, tb, g.M, g.N, g.K, kps, g.C, g.cm, g.cn, g.alpha, g.beta, g.C2, g.cm2, g.cn2, wsp,
+                                  errw);
+    return cudaGetLastError();
+  };
+  cudaError_t e;
+  if (split && (long long)gm * gn * splits >= 2 * sm_count)
+    e = launch(gemm_tf32_kernel<false, true, true>, Cfg<true, true>::SMEM_BYTES);
+  else if (split) e = launch(gemm_tf32_kernel<false, true, false>, Cfg<true>::SMEM_BYTES);
+  else e = launch(gemm_tf32_kernel<false, false, false>, Cfg<false>::SMEM_BYTES);
   if (e != cudaSuccess || splits == 1) return e;
   return splitk_reduce<float>(g, ws, splits, sm_count, st);
 }
