@@ -190,23 +190,28 @@ void einsum(Ctx<T>& cx, const Tn<const T>& A, const Tn<const T>& B, const Tn<T>&
       cudaError_t e = gemm_tf32(g, cx.ws, cx.ws_elems, cx.sm_count, nullptr, cx.st, true);
       if (e == cudaSuccess) return;
       if (e != cudaErrorNotSupported) GK(e);
-      // a large product whose operands TMA cannot load as they lie: copy them K-major first
+      // a large product one of whose operands TMA cannot load as it lies: copy that one K-major first
       // (O(size) against the O(M N K) of the product)
       if ((long long)g.M * g.N * g.K >= (1ll << 24) && g.K % 4 == 0 && cx.ar) {
-        const size_t na = (size_t)g.M * g.K, nb = (size_t)g.N * g.K;
-        if (na > cx.sa_n) cx.sa = cx.ar->template alloc<T>(na), cx.sa_n = na;
-        if (nb > cx.sb_n) cx.sb = cx.ar->template alloc<T>(nb), cx.sb_n = nb;
-        GK(copy_map<T, T>(g.M, g.K, g.A, g.am, g.ak, cx.sa, IdxMap::lin(g.K), IdxMap::lin(1), 1.0, cx.st));
-        GK(copy_map<T, T>(g.N, g.K, g.B, g.bn, g.bk, cx.sb, IdxMap::lin(g.K), IdxMap::lin(1), 1.0, cx.st));
         GemmArgs<T> h = g;
-        h.A = cx.sa;
-        h.am = IdxMap::lin(g.K);
-        h.ak = IdxMap::lin(1);
-        h.a_kfast = true;
-        h.B = cx.sb;
-        h.bn = IdxMap::lin(g.K);
-        h.bk = IdxMap::lin(1);
-        h.b_kfast = true;
+        if (!tf32_loadable(g.A, g.am, g.ak, g.K)) {
+          const size_t na = (size_t)g.M * g.K;
+          if (na > cx.sa_n) cx.sa = cx.ar->template alloc<T>(na), cx.sa_n = na;
+          GK(copy_map<T, T>(g.M, g.K, g.A, g.am, g.ak, cx.sa, IdxMap::lin(g.K), IdxMap::lin(1), 1.0, cx.st));
+          h.A = cx.sa;
+          h.am = IdxMap::lin(g.K);
+          h.ak = IdxMap::lin(1);
+          h.a_kfast = true;
+        }
+        if (!tf32_loadable(g.B, g.bn, g.bk, g.K)) {
+          const size_t nb = (size_t)g.N * g.K;
+          if (nb > cx.sb_n) cx.sb = cx.ar->template alloc<T>(nb), cx.sb_n = nb;
+          GK(copy_map<T, T>(g.N, g.K, g.B, g.bn, g.bk, cx.sb, IdxMap::lin(g.K), IdxMap::lin(1), 1.0, cx.st));
+          h.B = cx.sb;
+          h.bn = IdxMap::lin(g.K);
+          h.bk = IdxMap::lin(1);
+          h.b_kfast = true;
+        }
         e = gemm_tf32(h, cx.ws, cx.ws_elems, cx.sm_count, nullptr, cx.st, true);
         if (e == cudaSuccess) return;
         if (e != cudaErrorNotSupported) GK(e);

@@ -42,6 +42,8 @@ cudaError_t splitk_reduce(const GemmArgs<T>& g, const T* ws, int splits, int sm_
 cudaError_t gemm_tf32(const GemmArgs<float>& g, float* ws, size_t ws_elems, int sm_count, uint32_t* errw,
                       cudaStream_t st, bool split = false);
 
+bool tf32_loadable(const float* p, const IdxMap& rows, const IdxMap& k, int K);
+
 // FP64-class GEMM of double-FP32 operands on the tensor cores (fixed-point
 // digit split, exact FP32 accumulation of the leading digit levels), with TF32
 // digits (kind::tf32) or BF16 digits (kind::f16, bf16 = true); scratch as

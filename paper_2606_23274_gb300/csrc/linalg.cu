@@ -1514,8 +1514,18 @@ __global__ void __launch_bounds__(256) copy_map_tiled_kernel(int rows, int cols,
   }
 }
 
-// Whether the innermost level of a map steps through neighbouring memory.
-inline bool unit_inner(const IdxMap& m) { return m.s2 == 1; }
+// 32-byte sectors that 32 neighbouring indices of a map touch: what a warp along them costs.
+inline int map_sectors(const IdxMap& m, int n, int bytes) {
+  long long last[32];
+  int k = 0;
+  for (int i = 0; i < (n < 32 ? n : 32); ++i) {
+    const long long s = m(i) * bytes / 32;
+    int t = 0;
+    while (t < k && last[t] != s) ++t;
+    if (t == k) last[k++] = s;
+  }
+  return k;
+}
 
 template <typename Tin, typename Tout>
 cudaError_t copy_map(int rows, int cols, const Tin* in, IdxMap im, IdxMap in_, Tout* out, IdxMap om, IdxMap on,
@@ -1523,12 +1533,13 @@ cudaError_t copy_map(int rows, int cols, const Tin* in, IdxMap im, IdxMap in_, T
   long long tot = (long long)rows * cols;
   if (tot <= 0) return cudaSuccess;
   ++tl_launches;
-  // transposing copies from 32 x 32 on; below, and where both sides run along the columns (or neither runs
-  // along one), one thread an element; where both run along the rows (column-major copies), so do the threads
-  const bool rows_in = unit_inner(im) && !unit_inner(in_), cols_out = unit_inner(on) && !unit_inner(om);
-  const bool cols_in = unit_inner(in_) && !unit_inner(im), rows_out = unit_inner(om) && !unit_inner(on);
-  const bool tiled = rows >= 32 && cols >= 32 && ((rows_in && cols_out) || (cols_in && rows_out));
-  if ((tiled && cols_in) || (!tiled && rows_in && rows_out)) {  // swap the roles of rows and columns
+  // The direction, rows or columns, in which a warp touches fewer sectors, of the input and of the output. Where the
+  // two differ, 32 x 32 tiles (from 16 rows and columns on); else one thread an element, along that direction.
+  // A warp reads along the rows of the gradient's [a s z w b t] operand at 8 sectors, along its columns at 16 to 32.
+  const bool rows_in = rows > 1 && (cols == 1 || map_sectors(im, rows, sizeof(Tin)) < map_sectors(in_, cols, sizeof(Tin)));
+  const bool rows_out = rows > 1 && (cols == 1 || map_sectors(om, rows, sizeof(Tout)) < map_sectors(on, cols, sizeof(Tout)));
+  const bool tiled = rows >= 16 && cols >= 16 && rows_in != rows_out;
+  if (tiled ? rows_out : rows_in && rows_out) {  // swap the roles of rows and columns
     std::swap(rows, cols);
     std::swap(im, in_);
     std::swap(om, on);
