@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(NT, 3) gemm_simt_kernel(GemmArgs<T> g, T* __re
       Bs[kk][r] = w;
     }
     __syncthreads();
-#pragma unroll
+#pragma unroll(MT == 1 ? 8 : 4)
     for (int kk = 0; kk < BK; ++kk) {
       T a[MT], b[MT];
 #pragma unroll
@@ -85,46 +85,57 @@ __global__ void __launch_bounds__(NT, 3) gemm_simt_kernel(GemmArgs<T> g, T* __re
     }
     return;
   }
+  // output offsets of the tile's rows and columns: one evaluation each, one copy of each map's code
+  __syncthreads();
+  __shared__ long long crow2[TB], ccol2[TB];
+  if (tid < TB) arow[tid] = g.cm(min(m0 + tid, g.M - 1));
+  else if (tid < 2 * TB) brow[tid - TB] = g.cn(min(n0 + tid - TB, g.N - 1));
+  if (g.C2) {
+    if (tid < TB) crow2[tid] = g.cm2(min(m0 + tid, g.M - 1));
+    else if (tid < 2 * TB) ccol2[tid - TB] = g.cn2(min(n0 + tid - TB, g.N - 1));
+  }
+  __syncthreads();
 #pragma unroll
   for (int i = 0; i < MT; ++i) {
-    int m = m0 + ty + 16 * i;
-    if (m >= g.M) continue;
-    long long cr = g.cm(m);
-    long long cr2 = g.C2 ? g.cm2(m) : 0;
+    const int ml = ty + 16 * i;
+    if (m0 + ml >= g.M) continue;
 #pragma unroll
     for (int j = 0; j < MT; ++j) {
-      int n = n0 + tx + 16 * j;
-      if (n >= g.N) continue;
-      long long o = cr + g.cn(n);
+      const int nl = tx + 16 * j;
+      if (n0 + nl >= g.N) continue;
       T v = g.alpha * acc[i][j];
-      if (g.C2) g.C2[cr2 + g.cn2(n)] = v;
-      if (g.beta != T(0)) v += g.beta * g.C[o];
-      g.C[o] = v;
+      if (g.C2) g.C2[crow2[ml] + ccol2[nl]] = v;
+      T* o = g.C + (arow[ml] + brow[nl]);
+      if (g.beta != T(0)) v += g.beta * *o;
+      *o = v;
     }
   }
 }
 
 // FP32. 128 threads, each 8 x 4 outputs (rows 8 ty .. 8 ty + 7, columns tx + TX j); k-tiles of 16 in two shared
-// buffers, the next one's loads in registers while the present one is multiplied, and the k offsets of 256 terms
-// tabulated at a time. The kernel above waits for its loads and evaluates the k maps in every k-tile: for the
-// gradient's products (3072 x 384 x 96, 6144 x 192 x 192, 9216 x 32 x 128) it was bound by that latency, at
-// 5 TFLOP/s. Sums run in the same order, so the results are the same bits.
+// buffers, the next one's loads in registers while the present one is multiplied, the offsets of 256 terms of K
+// tabulated at a time. The code is kept short: the loads and each index map stand once, the products are unrolled by
+// 4, and the outputs go through shared memory to one small loop, which also writes them along their fast direction.
+// A few warps an SM cannot hide the fetch of long straight code: with the outputs unrolled (bounds, second copy, beta)
+// a 64 x 64 x 16 product took 8.2 us, and the products of the gradient (3072 x 384 x 96, ...) three times their
+// arithmetic.
 template <int BM, int BN>
 __global__ void __launch_bounds__(128) gemm_f32_kernel(GemmArgs<float> g, float* __restrict__ ws, int k_per_split) {
-  constexpr int TX = BN / 4, KC = 256, NA = BM * BK / 128, NB = BN * BK / 128;
-  static_assert(TX * (BM / 8) == 128, "8 x 4 outputs a thread");
-  __shared__ __align__(16) float As[2][BK][BM + 4];
-  __shared__ float Bs[2][BK][BN + 1];
+  constexpr int NTH = 128, TX = BN / 4, KC = 256, NA = BM * BK / NTH, NB = BN * BK / NTH;
+  constexpr int LA = BM + 4, LB = BN + 1, SA = BK * LA, SB = BK * LB;
+  static_assert(TX * (BM / 8) == NTH, "8 x 4 outputs a thread");
+  static_assert(2 * (SA + SB) >= BM * (BN + 1), "the output tile takes the place of the operands");
+  __shared__ __align__(16) float sm[2 * (SA + SB)];  // [2][BK][LA] of A, [2][BK][LB] of B; then [BM][BN + 1] of C
   __shared__ long long arow[BM], brow[BN];
   __shared__ long long akoff[KC], bkoff[KC];
   const int tid = threadIdx.x;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int kb = blockIdx.z * k_per_split;
   const int ke = min(g.K, kb + k_per_split);
-  for (int t = tid; t < BM + BN; t += 128) {
-    if (t < BM) arow[t] = (m0 + t < g.M) ? g.am(m0 + t) : 0;
-    else brow[t - BM] = (n0 + t - BM < g.N) ? g.bn(n0 + t - BM) : 0;
-  }
+#pragma unroll 1
+  for (int t = tid; t < BM; t += NTH) arow[t] = (m0 + t < g.M) ? g.am(m0 + t) : 0;
+#pragma unroll 1
+  for (int t = tid; t < BN; t += NTH) brow[t] = (n0 + t < g.N) ? g.bn(n0 + t) : 0;
   const int tx = tid % TX, ty = tid / TX;
   float acc[8][4];
 #pragma unroll
@@ -132,102 +143,106 @@ __global__ void __launch_bounds__(128) gemm_f32_kernel(GemmArgs<float> g, float*
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
   float ra[NA], rb[NB];
-  auto load = [&](int k0) {
-    const int c0 = (k0 - kb) % KC;
-    if (c0 == 0) {  // the next stretch of k offsets
-      __syncthreads();
-      for (int t = tid; t < KC; t += 128) {
-        akoff[t] = k0 + t < ke ? g.ak(k0 + t) : 0;
-        bkoff[t] = k0 + t < ke ? g.bk(k0 + t) : 0;
+  int buf = 0;
+#pragma unroll 1
+  for (int k0 = kb - BK; k0 < ke; k0 += BK) {  // the first pass only loads
+    const int kn = k0 + BK;                    // the k-tile to load
+    if (kn < ke) {
+      const int c0 = (kn - kb) % KC;
+      if (c0 == 0) {  // the next stretch of k offsets
+        __syncthreads();
+        const int cnt = min(KC, (ke - kn + BK - 1) / BK * BK);
+#pragma unroll 1
+        for (int t = tid; t < cnt; t += NTH) {
+          akoff[t] = kn + t < ke ? g.ak(kn + t) : 0;
+          bkoff[t] = kn + t < ke ? g.bk(kn + t) : 0;
+        }
+        __syncthreads();
       }
-      __syncthreads();
-    }
 #pragma unroll
-    for (int i = 0; i < NA; ++i) {
-      const int e = tid + 128 * i;
-      const int r = g.a_kfast ? e / BK : e % BM, kk = g.a_kfast ? e % BK : e / BM;
-      ra[i] = (m0 + r < g.M && k0 + kk < ke) ? g.A[arow[r] + akoff[c0 + kk]] : 0.f;
-    }
+      for (int i = 0; i < NA; ++i) {
+        const int e = tid + NTH * i;
+        const int r = g.a_kfast ? e / BK : e % BM, kk = g.a_kfast ? e % BK : e / BM;
+        ra[i] = (m0 + r < g.M && kn + kk < ke) ? g.A[arow[r] + akoff[c0 + kk]] : 0.f;
+      }
 #pragma unroll
-    for (int i = 0; i < NB; ++i) {
-      const int e = tid + 128 * i;
-      const int r = g.b_kfast ? e / BK : e % BN, kk = g.b_kfast ? e % BK : e / BN;
-      rb[i] = (n0 + r < g.N && k0 + kk < ke) ? g.B[brow[r] + bkoff[c0 + kk]] : 0.f;
+      for (int i = 0; i < NB; ++i) {
+        const int e = tid + NTH * i;
+        const int r = g.b_kfast ? e / BK : e % BN, kk = g.b_kfast ? e % BK : e / BN;
+        rb[i] = (n0 + r < g.N && kn + kk < ke) ? g.B[brow[r] + bkoff[c0 + kk]] : 0.f;
+      }
     }
-  };
-  auto store = [&](int buf) {
-#pragma unroll
-    for (int i = 0; i < NA; ++i) {
-      const int e = tid + 128 * i;
-      const int r = g.a_kfast ? e / BK : e % BM, kk = g.a_kfast ? e % BK : e / BM;
-      As[buf][kk][r] = ra[i];
-    }
-#pragma unroll
-    for (int i = 0; i < NB; ++i) {
-      const int e = tid + 128 * i;
-      const int r = g.b_kfast ? e / BK : e % BN, kk = g.b_kfast ? e % BK : e / BN;
-      Bs[buf][kk][r] = rb[i];
-    }
-  };
-  if (kb < ke) {
-    load(kb);
-    store(0);
-    __syncthreads();
-    int buf = 0;
-    for (int k0 = kb; k0 < ke; k0 += BK) {
-      const bool more = k0 + BK < ke;
-      if (more) load(k0 + BK);
-#pragma unroll
+    if (k0 >= kb) {
+      const float* As = sm + buf * SA + 8 * ty;
+      const float* Bs = sm + 2 * SA + buf * SB + tx;
+#pragma unroll 4
       for (int kk = 0; kk < BK; ++kk) {
-        const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][8 * ty]);
-        const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][8 * ty + 4]);
-        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-        float b[4];
+        float a[8], b[4];
+        *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(As + kk * LA);
+        *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(As + kk * LA + 4);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[buf][kk][tx + TX * j];
+        for (int j = 0; j < 4; ++j) b[j] = Bs[kk * LB + TX * j];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
           for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
       }
-      if (more) store(buf ^ 1);
-      buf ^= 1;
-      __syncthreads();
     }
-  }
-  if (ws) {  // split-K partial: dense [split][M][N]
-    float* w = ws + (size_t)blockIdx.z * g.M * g.N;
+    buf ^= 1;
+    if (kn < ke) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int m = m0 + 8 * ty + i;
-      if (m >= g.M) continue;
+      for (int i = 0; i < NA; ++i) {
+        const int e = tid + NTH * i;
+        const int r = g.a_kfast ? e / BK : e % BM, kk = g.a_kfast ? e % BK : e / BM;
+        sm[buf * SA + kk * LA + r] = ra[i];
+      }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int n = n0 + tx + TX * j;
-        if (n < g.N) w[(size_t)m * g.N + n] = acc[i][j];
+      for (int i = 0; i < NB; ++i) {
+        const int e = tid + NTH * i;
+        const int r = g.b_kfast ? e / BK : e % BN, kk = g.b_kfast ? e % BK : e / BN;
+        sm[2 * SA + buf * SB + kk * LB + r] = rb[i];
       }
     }
-    return;
-  }
-  long long cn[4], cn2[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int n = min(n0 + tx + TX * j, g.N - 1);
-    cn[j] = g.cn(n);
-    cn2[j] = g.C2 ? g.cn2(n) : 0;
+    __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int m = m0 + 8 * ty + i;
-    if (m >= g.M) continue;
-    const long long cr = g.cm(m), cr2 = g.C2 ? g.cm2(m) : 0;
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (n0 + tx + TX * j >= g.N) continue;
-      float v = g.alpha * acc[i][j];
-      if (g.C2) g.C2[cr2 + cn2[j]] = v;
-      if (g.beta != 0.f) v += g.beta * g.C[cr + cn[j]];
-      g.C[cr + cn[j]] = v;
+    for (int j = 0; j < 4; ++j) sm[(8 * ty + i) * (BN + 1) + tx + TX * j] = acc[i][j];
+  // output offsets of the tile's rows and columns, in the tables that are free now (split-K partials: dense [M][N])
+#pragma unroll 1
+  for (int t = tid; t < BM; t += NTH) {
+    const int m = min(m0 + t, g.M - 1);
+    arow[t] = ws ? (long long)m * g.N : g.cm(m);
+    if (g.C2) akoff[t] = g.cm2(m);
+  }
+#pragma unroll 1
+  for (int t = tid; t < BN; t += NTH) {
+    const int n = min(n0 + t, g.N - 1);
+    brow[t] = ws ? n : g.cn(n);
+    if (g.C2) bkoff[t] = g.cn2(n);
+  }
+  __syncthreads();
+  const int mh = min(BM, g.M - m0), nh = min(BN, g.N - n0);
+  float* out = ws ? ws + (size_t)blockIdx.z * g.M * g.N : g.C;
+  const float alpha = ws ? 1.f : g.alpha, beta = ws ? 0.f : g.beta;
+  const bool by_rows = !ws && g.cn.s2 != 1 && g.cm.s2 == 1;  // neighbouring threads take neighbouring rows
+#pragma unroll 4
+  for (int e = tid; e < BM * BN; e += NTH) {
+    const int ml = by_rows ? e % BM : e / BN, nl = by_rows ? e / BM : e % BN;
+    if (ml < mh && nl < nh) {
+      float v = alpha * sm[ml * (BN + 1) + nl];
+      float* o = out + (arow[ml] + brow[nl]);
+      if (beta != 0.f) v += beta * *o;
+      *o = v;
+    }
+  }
+  if (g.C2 && !ws) {
+    const bool rows2 = g.cn2.s2 != 1 && g.cm2.s2 == 1;
+#pragma unroll 4
+    for (int e = tid; e < BM * BN; e += NTH) {
+      const int ml = rows2 ? e % BM : e / BN, nl = rows2 ? e / BM : e % BN;
+      if (ml < mh && nl < nh) g.C2[akoff[ml] + bkoff[nl]] = alpha * sm[ml * (BN + 1) + nl];
     }
   }
 }
