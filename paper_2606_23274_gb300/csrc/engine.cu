@@ -933,7 +933,9 @@ int factorize_body(tt_fit* h, int m, int n, int sweep, int site1, int need) {
     if constexpr (std::is_same<F, double>::value) {
       // on R2^T, whose columns are graded (see svd_tall64): R2^T = Vr S Ur^T
       copymap<F, F>(h, ks, ks, fR2, IdxMap::lin(1), IdxMap::lin(ks), fX, IdxMap::lin(ks), IdxMap::lin(1));
-      jac(ks, ks, fX, fV, fS, fU);
+      const cudaError_t e = svd_graded64(ks, fX, fV, fS, fU, fBt, fOm, 60, W(h).errw, h->sm_count, W(h).st);
+      if (e == cudaErrorNotSupported) jac(ks, ks, fX, fV, fS, fU);
+      else CK(e);
     } else {
       jac(ks, ks, fR2, fU, fS, fV);               // R2 = Ur S Vr^T
     }
@@ -965,7 +967,7 @@ int factorize_body(tt_fit* h, int m, int n, int sweep, int site1, int need) {
   else copymap<F, F>(h, m, n, MF, IdxMap::lin(n), IdxMap::lin(1), fX, IdxMap::lin(1), IdxMap::lin(m));
   F* Ufull;
   if constexpr (std::is_same<F, double>::value) {
-    CK(svd_tall64(q, p, fX, fQ, fVw, &Ufull, fS, fV, 60, W(h).errw, h->sm_count, W(h).st));
+    CK(svd_tall64(q, p, fX, fQ, fVw, fU, fR2, &Ufull, fS, fV, 60, W(h).errw, h->sm_count, W(h).st));
   } else if (q > p) {
     qrf(q, p, fX, fQ, fR);                        // X = Qx Rx
     jac(p, p, fR, fU, fS, fV);                    // Rx = Ur S Vr^T
@@ -2055,8 +2057,9 @@ void zipup_rl(tt_fit* h, const ZipArgs& z, std::vector<double*>& C, std::vector<
   T *Y = take(sz_nk), *Q = take(sz_nk), *Rq = take((size_t)ks * ks), *Z = take(sz_z), *Zc = take(sz_zc);
   T *Ux = take(sz_u), *Sv = take(sz_p), *Vx = take(sz_pp), *Vw = take(sz_pp), *Vn = take(std::max(sz_nk, sz_mn));
   T *Rc = take(sz_r), *Rn = take(sz_r), *ws = take(wse);
-  T *Al = nullptr, *Bl = nullptr;
+  T *Al = nullptr, *Bl = nullptr, *E0 = nullptr, *E1 = nullptr;
   if (!std::is_same<T, double>::value) Al = take(sz_ab), Bl = take(sz_ab);
+  else E0 = take(sz_pp), E1 = take(sz_pp);  // scratch of the FP64 decomposition
   {  // R_{L+1} = [[[1]]]
     const T one = T(1);
     CK(cudaMemcpyAsync(Rc, &one, sizeof(T), cudaMemcpyHostToDevice, st));
@@ -2192,7 +2195,7 @@ void zipup_rl(tt_fit* h, const ZipArgs& z, std::vector<double*>& C, std::vector<
     auto zsvd = [&](int q, int pc, T* T1, T* V) -> T* {
       if constexpr (std::is_same<T, double>::value) {
         T* U = nullptr;
-        CK(svd_tall64(q, pc, Zc, T1, Vw, &U, Sv, V, 60, w.errw, h->sm_count, st));
+        CK(svd_tall64(q, pc, Zc, T1, Vw, E0, E1, &U, Sv, V, 60, w.errw, h->sm_count, st));
         return U;
       } else {
         CK(jacobi_svd<T, T>(q, pc, Zc, T1, Sv, V, Vw, 60, w.errw, st));

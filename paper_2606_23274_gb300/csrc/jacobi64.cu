@@ -143,8 +143,8 @@ __host__ __device__ inline int jacobi64_ld(int q, int p, bool want_v) {
 
 template <int LP, bool SCALED>
 __global__ void __launch_bounds__(1024)
-    jacobi64_kernel(int q, int p, int b, const double* __restrict__ Win, int max_sweeps, double tol, uint32_t* errw,
-                    double* __restrict__ Uo, double* __restrict__ So, double* __restrict__ Vo) {
+    jacobi64_kernel(int q, int p, int b, const double* Win, const double* Vin, int max_sweeps, double tol,
+                    uint32_t* errw, double* Uo, double* __restrict__ So, double* Vo) {
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), NC = (int)cl.num_blocks();
   const int P = 2 * NC;
@@ -174,7 +174,9 @@ __global__ void __launch_bounds__(1024)
       for (int r = threadIdx.x; r < ld; r += blockDim.x) {
         double v = 0.0;
         if (r == ld - 3 || r == ld - 2) v = 1.0;
-        else if (gid < p) v = r < q ? Win[(size_t)gid * q + r] : ((r >= qs && r - qs == gid && r < ld - J64_TAIL) ? 1.0 : 0.0);
+        else if (gid < p && r < q) v = Win[(size_t)gid * q + r];
+        else if (gid < p && r >= qs && r - qs < p && r < ld - J64_TAIL)
+          v = Vin ? Vin[(size_t)gid * p + r - qs] : (r - qs == gid ? 1.0 : 0.0);
         x[r] = v;
       }
     }
@@ -314,7 +316,8 @@ inline size_t jacobi64_smem(int q, int p, bool want_v, int nc) {
 // pay from 300 rows on (256 x 74: 5.3 ms against 5.6 ms; 128 x 128: 8.2 against 7.9).
 namespace {
 
-using Jacobi64Kernel = void (*)(int, int, int, const double*, int, double, uint32_t*, double*, double*, double*);
+using Jacobi64Kernel = void (*)(int, int, int, const double*, const double*, int, double, uint32_t*, double*, double*,
+                                double*);
 
 struct Jacobi64Plan {
   Jacobi64Kernel kern = nullptr;  // null: does not fit
@@ -367,24 +370,77 @@ cudaError_t jacobi64_plan(int q, int p, bool want_v, cudaStream_t st, Jacobi64Pl
 
 }  // namespace
 
-cudaError_t jacobi_svd64(int q, int p, const double* W, double* U, double* Sv, double* V, int max_sweeps,
-                         uint32_t* errw, cudaStream_t st) {
+cudaError_t jacobi_svd64(int q, int p, const double* W, const double* Vin, double* U, double* Sv, double* V,
+                         int max_sweeps, uint32_t* errw, cudaStream_t st) {
   const double tol = 4.0 * DBL_EPSILON * sqrt((double)q);  // as in jacobi_svd
   Jacobi64Plan plan;
   cudaError_t e = jacobi64_plan(q, p, V != nullptr, st, plan);
   if (e != cudaSuccess) return e;
   if (!plan.kern) return cudaErrorNotSupported;
   ++tl_launches;
-  e = cudaLaunchKernelEx(&plan.cfg, plan.kern, q, p, plan.b, W, max_sweeps, tol, errw, U, Sv, V);
+  e = cudaLaunchKernelEx(&plan.cfg, plan.kern, q, p, plan.b, W, Vin, max_sweeps, tol, errw, U, Sv, V);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// SVD of a p x p matrix with graded columns, L = U diag(S) W^T.
+// Four fifths of the sweeps run in FP32, where they cost a quarter: an FP32 Jacobi of L gives rotations W0, made
+// orthonormal to FP64 rounding by two Newton-Schulz steps, and the FP64 Jacobi of L W0 needs 3 or 4 sweeps for its own
+// stopping rule instead of 10 (spectra down to 1e-18 s_1: the columns are graded, so FP32 keeps each to its own
+// rounding). The result is as accurate as without: every rotation that counts is taken in FP64.
+// U must not be L; e0, e1: p x p scratch each, or null (no room: all sweeps in FP64).
+// 128 x 128: 3.3 ms by FP64 sweeps alone.
+cudaError_t svd_graded64(int p, const double* L, double* U, double* Sv, double* W, double* e0, double* e1, int max_sweeps,
+                         uint32_t* errw, int sm_count, cudaStream_t st) {
+  Jacobi64Plan plan;
+  cudaError_t e = jacobi64_plan(p, p, true, st, plan);
+  if (e != cudaSuccess) return e;
+  if (!plan.kern) return cudaErrorNotSupported;
+  if (p < 32 || !e0 || !e1 || !jacobi32_rotations_fits(p))
+    return jacobi_svd64(p, p, L, nullptr, U, Sv, W, max_sweeps, errw, st);
+  const long long n = (long long)p * p;
+  double* t = U;  // scratch until the decomposition writes it
+  float *L32 = (float*)t, *V32 = L32 + n;
+  int* ex = (int*)Sv;  // free until the decomposition writes it
+  if ((e = absmax_exponent<double>(L, n, ex, st)) != cudaSuccess) return e;
+  if ((e = copy_pow2<double, float>(n, L, L32, ex, st)) != cudaSuccess) return e;
+  if ((e = jacobi32_rotations(p, L32, V32, 8, st)) != cudaSuccess) return e;
+  const IdxMap one = IdxMap::lin(1), row = IdxMap::lin(p), zero = IdxMap::lin(0);
+  if ((e = copy_map<float, double>(1, (int)n, V32, zero, one, W, zero, one, 1.0, st)) != cudaSuccess) return e;
+  double *X = W, *Xn = e1;
+  for (int it = 0; it < 2; ++it) {  // X <- X (3 I - X^T X) / 2
+    GemmArgs<double> g;
+    g.M = g.N = g.K = p;
+    g.A = X; g.am = row; g.ak = one;
+    g.B = X; g.bn = row; g.bk = one;
+    g.C = e0; g.cm = one; g.cn = row;
+    if ((e = gemm_simt<double>(g, nullptr, 0, sm_count, st)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(Xn, X, sizeof(double) * n, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+    GemmArgs<double> a;
+    a.M = a.N = a.K = p;
+    a.A = X; a.am = one; a.ak = row; a.a_kfast = false;
+    a.B = e0; a.bn = row; a.bk = one;
+    a.C = Xn; a.cm = one; a.cn = row;
+    a.alpha = -0.5;
+    a.beta = 1.5;
+    if ((e = gemm_simt<double>(a, nullptr, 0, sm_count, st)) != cudaSuccess) return e;
+    std::swap(X, Xn);
+  }
+  GemmArgs<double> g;  // t = L W0 (W0 is back in W)
+  g.M = g.N = g.K = p;
+  g.A = L; g.am = one; g.ak = row; g.a_kfast = false;
+  g.B = W; g.bn = row; g.bk = one;
+  g.C = t; g.cm = one; g.cn = row;
+  if ((e = gemm_simt<double>(g, nullptr, 0, sm_count, st)) != cudaSuccess) return e;
+  // outputs may take the inputs' place: the kernel reads both before its first barrier and writes after its last sweep
+  return jacobi_svd64(p, p, t, W, U, Sv, W, max_sweeps, errw, st);
 }
 
 // The same decomposition by way of X = Q R: Jacobi on R^T, whose columns come graded (row i of R is of the
 // size of the i-th singular value), R^T = U' S W^T, so that X = (Q W) S U'^T. On the square or tall matrix
 // itself the columns are of one size and Jacobi needs two to four times the sweeps (128 x 128, spectrum
 // 1 .. 1e-4: 22 against 9; 1 .. 1e-14: 36 against 10). Below 32 columns the QR costs what it saves.
-cudaError_t svd_tall64(int q, int p, double* X, double* T1, double* T2, double** U, double* Sv, double* V,
-                       int max_sweeps, uint32_t* errw, int sm_count, cudaStream_t st) {
+cudaError_t svd_tall64(int q, int p, double* X, double* T1, double* T2, double* e0, double* e1, double** U,
+                       double* Sv, double* V, int max_sweeps, uint32_t* errw, int sm_count, cudaStream_t st) {
   *U = T1;
   if (q <= 0 || p <= 0) return cudaSuccess;
   Jacobi64Plan plan;
@@ -395,7 +451,7 @@ cudaError_t svd_tall64(int q, int p, double* X, double* T1, double* T2, double**
   if (e != cudaSuccess) return e;
   const IdxMap one = IdxMap::lin(1), row = IdxMap::lin(p);
   if ((e = copy_map<double, double>(p, p, T2, one, row, X, row, one, 1.0, st)) != cudaSuccess) return e;
-  if ((e = jacobi_svd64(p, p, X, V, Sv, T2, max_sweeps, errw, st)) != cudaSuccess) return e;
+  if ((e = svd_graded64(p, X, V, Sv, T2, e0, e1, max_sweeps, errw, sm_count, st)) != cudaSuccess) return e;
   GemmArgs<double> g;  // U = Q W
   g.M = q; g.N = p; g.K = p;
   g.A = T1; g.am = one; g.ak = IdxMap::lin(q); g.a_kfast = false;

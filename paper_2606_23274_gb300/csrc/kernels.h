@@ -89,13 +89,24 @@ cudaError_t jacobi_svd(int q, int p, S* W, S* U, S* Sv, S* V, S* Vwork, int max_
 
 // The FP64 decomposition on a cluster (jacobi64.cu), which jacobi_svd takes where it
 // fits; cudaErrorNotSupported otherwise. W is not changed.
-cudaError_t jacobi_svd64(int q, int p, const double* W, double* U, double* Sv, double* V, int max_sweeps,
-                         uint32_t* errw, cudaStream_t st);
+// Vin: rotations applied to W before (null: none), so that V = Vin times its own.
+cudaError_t jacobi_svd64(int q, int p, const double* W, const double* Vin, double* U, double* Sv, double* V,
+                         int max_sweeps, uint32_t* errw, cudaStream_t st);
+
+// At most `sweeps` sweeps of an FP32 Jacobi on the p x p W: its accumulated rotations V, columns of W V in
+// descending norm (jacobi32.cu). p limited: jacobi32_rotations_fits.
+bool jacobi32_rotations_fits(int p);
+cudaError_t jacobi32_rotations(int p, const float* W, float* V, int sweeps, cudaStream_t st);
+
+// SVD L = U diag(S) W^T of a p x p matrix with graded columns (jacobi64.cu).
+cudaError_t svd_graded64(int p, const double* L, double* U, double* Sv, double* W, double* e0, double* e1, int max_sweeps,
+                         uint32_t* errw, int sm_count, cudaStream_t st);
 
 // SVD of the q x p column-major X (q >= p; overwritten) as jacobi_svd<double> gives it, by way of a QR
-// where that saves sweeps. T1 (q x p), T2 (p x p): scratch. *U: where the left factor is, X or T1.
-cudaError_t svd_tall64(int q, int p, double* X, double* T1, double* T2, double** U, double* Sv, double* V,
-                       int max_sweeps, uint32_t* errw, int sm_count, cudaStream_t st);
+// where that saves sweeps. T1 (q x p), T2 (p x p), e0, e1 (p x p or null: see svd_graded64): scratch. *U: where
+// the left factor is, X or T1.
+cudaError_t svd_tall64(int q, int p, double* X, double* T1, double* T2, double* e0, double* e1, double** U, double* Sv,
+                       double* V, int max_sweeps, uint32_t* errw, int sm_count, cudaStream_t st);
 
 // ||X||_F of n values (type T) into *out (double), flags non-finite values.
 template <typename T>

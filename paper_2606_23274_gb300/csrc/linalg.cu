@@ -739,16 +739,6 @@ template cudaError_t qr_householder<float, float>(int, int, float*, float*, floa
 // round applies P/2 disjoint plane rotations that orthogonalise column pairs;
 // a sweep is P-1 rounds; it stops after a sweep without rotations.
 // ---------------------------------------------------------------------------
-// 1/sqrt(x) for x in [1, 2]: the hardware estimate refined by one Newton step
-// r <- r + r (1 - x r^2) / 2, so that cs^2 + sn^2 = cs^2 (1 + t^2) is 1 to the
-// FP32 rounding. An estimate left unrefined makes every rotation a rotation
-// times sqrt(cs^2 + sn^2), and the accumulated right factor drifts away from
-// orthonormal over the thousands of rotations of a decomposition.
-__device__ __forceinline__ float rot_rsqrt(float x) {
-  const float r = rsqrtf(x);
-  return fmaf(0.5f * r, fmaf(-x * r, r, 1.f), r);
-}
-
 // Jacobi rotation (c, s) that zeroes the (i, j) entry of the 2x2 Gram block
 // [[a, g], [g, b]] (Rutishauser's formulas). In FP32 the fast division serves
 // for the angle: any rotation this close to the exact one still drives the
@@ -1186,7 +1176,7 @@ cudaError_t jacobi_svd(int q, int p, S* W, S* U, S* Sv, S* V, S* Vwork, int max_
   const double eps = (sizeof(C) == 8) ? DBL_EPSILON : (double)FLT_EPSILON;
   const double tol = 4.0 * eps * sqrt((double)q);
   if constexpr (std::is_same<C, double>::value && std::is_same<S, double>::value) {
-    const cudaError_t e = jacobi_svd64(q, p, W, U, Sv, V, max_sweeps, errw, st);
+    const cudaError_t e = jacobi_svd64(q, p, W, nullptr, U, Sv, V, max_sweeps, errw, st);
     if (e != cudaErrorNotSupported) return e;  // otherwise the one-CTA kernel below
   }
   // the cluster kernel spreads the columns over JC SMs when there are enough of them (16, an

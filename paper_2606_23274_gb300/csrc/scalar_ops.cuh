@@ -1,4 +1,4 @@
-// Element operations of the Householder QR kernels in float, double and df32 arithmetic.
+// Element operations of the Householder QR and Jacobi kernels.
 #pragma once
 #include "common.cuh"
 
@@ -51,6 +51,16 @@ __device__ __forceinline__ C qshfl(C v, int src) {
 template <>
 __device__ __forceinline__ df32 qshfl<df32>(df32 v, int src) {
   return df32(__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src));
+}
+
+// 1/sqrt(x) for x in [1, 2]: the hardware estimate refined by one Newton step
+// r <- r + r (1 - x r^2) / 2, so that cs^2 + sn^2 = cs^2 (1 + t^2) is 1 to the
+// FP32 rounding. An estimate left unrefined makes every rotation a rotation
+// times sqrt(cs^2 + sn^2), and the accumulated right factor drifts away from
+// orthonormal over the thousands of rotations of a decomposition.
+__device__ __forceinline__ float rot_rsqrt(float x) {
+  const float r = rsqrtf(x);
+  return fmaf(0.5f * r, fmaf(-x * r, r, 1.f), r);
 }
 
 }  // namespace ttfit

@@ -45,7 +45,7 @@ __global__ void svd_outputs_kernel(int m, int n, int tr, const double* __restric
 }
 
 cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, double* U, double* S, double* Vt,
-                    int* k_dev, double* scratch, cudaStream_t st) {
+                    int* k_dev, double* scratch, double* extra, cudaStream_t st) {
   const int r = std::min(m, n), q = std::max(m, n);
   const bool tr = m < n;
   double* X = scratch;
@@ -66,7 +66,7 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = svd_tall64(q, r, X, Ux, Vw, &Ux, Sv, Vx, 60, info, sms, st)) != cudaSuccess) return e;
+  if ((e = svd_tall64(q, r, X, Ux, Vw, extra, extra ? extra + (size_t)r * r : nullptr, &Ux, Sv, Vx, 60, info, sms, st)) != cudaSuccess) return e;
   if ((e = fix_signs<double>(tr ? r : q, tr ? q : r, r, tr ? Vx : Ux, tr ? r : q, tr ? Ux : Vx, tr ? q : r, st)) !=
       cudaSuccess)
     return e;
@@ -93,17 +93,17 @@ extern "C" tt_status tt_svd_truncated(const double* M, int m, int n, int chi_max
   tt_status s = svd_check(M, m, n, chi_max, tau_rel, U, S, Vt, k_out);
   if (s != TT_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
-  const size_t nd = svd_scratch_doubles(m, n);
+  const size_t nd = svd_scratch_doubles(m, n), r2 = (size_t)std::min(m, n) * std::min(m, n);
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return TT_ERR_CUDA;
   }
   size_t got = 0;
-  double* scratch = (double*)block_take(dev, nd * sizeof(double), &got);
+  double* scratch = (double*)block_take(dev, (nd + 2 * r2) * sizeof(double), &got);
   if (!scratch) return TT_ERR_OUT_OF_MEMORY;
   int* k_dev = (int*)(scratch + nd - 1);
-  cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, k_dev, scratch, st);
+  cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, k_dev, scratch, scratch + nd, st);
   int k = 0;
   uint32_t flags[2] = {0, 0};
   if (e == cudaSuccess) e = cudaMemcpyAsync(&k, k_dev, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -167,9 +167,12 @@ extern "C" tt_status tt_svd_truncated_noalloc(const double* M, int m, int n, int
     return TT_ERR_CUDA;
   }
   int* k_dev = (int*)(scratch + nd - 1);
+  // the FP32 sweeps' scratch, where the array has room for it as well
+  const size_t r = std::min(m, n);
+  double* extra = nd + 2 * r * r <= kNoAllocDoubles ? scratch + nd : nullptr;
   // svd_run clears the error flags it reads; every other scratch word it uses
   // is written before it is read
-  cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, k_dev, scratch, st);
+  cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, k_dev, scratch, extra, st);
   int k = 0;
   uint32_t flags[2] = {0, 0};
   if (e == cudaSuccess) e = cudaMemcpyAsync(&k, k_dev, sizeof(int), cudaMemcpyDeviceToHost, st);

@@ -30,3 +30,25 @@ def test_svd_at_the_edges_of_the_kernels(m, n, floor):
     assert np.linalg.norm(U * S[None, :] @ Vt - M) <= tol * norm
     assert np.abs(U.T @ U - np.eye(r)).max() <= tol and np.abs(Vt @ Vt.T - np.eye(r)).max() <= tol
     assert np.abs(S - np.linalg.svd(M, compute_uv=False)).max() <= tol * norm
+
+
+@pytest.mark.parametrize("r,floor", [(32, 1e-4), (33, 1e-14), (64, 1e-18), (95, 1e-9), (96, 1e-14), (128, 1e-4), (129, 1e-14),
+                                     (193, 1e-6), (256, 1e-3)])
+def test_svd_with_fp32_sweeps_is_as_accurate(r, floor):
+    """From 32 columns on the early sweeps run in FP32: clustered, graded and rank-deficient spectra still come out
+    to FP64 rounding."""
+    rng = np.random.default_rng(r)
+    s = floor ** (np.arange(r) / (r - 1))
+    s[r // 3:r // 3 + 4] = s[r // 3]        # a cluster
+    s[-2:] = 0.0                            # rank deficient
+    Q1, _ = np.linalg.qr(rng.standard_normal((r, r)))
+    Q2, _ = np.linalg.qr(rng.standard_normal((r, r)))
+    M = (Q1 * s) @ Q2.T
+    U, S, Vt, _ = ttfit.tt_svd_truncated(M, chi_max=r, tau_rel=0.0)
+    U, S, Vt = U.cpu().numpy(), S.cpu().numpy(), Vt.cpu().numpy()
+    tol = 60 * r * EPS
+    k = int(np.sum(s > 1e-9))               # vectors of values above the rounding level of the product M
+    assert np.linalg.norm(U * S[None, :] @ Vt - M) <= tol * np.linalg.norm(M)
+    assert np.abs(U[:, :k].T @ U[:, :k] - np.eye(k)).max() <= tol
+    assert np.abs(Vt[:k] @ Vt[:k].T - np.eye(k)).max() <= tol
+    assert np.abs(S - s[np.argsort(-s)]).max() <= tol
