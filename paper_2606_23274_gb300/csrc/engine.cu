@@ -240,7 +240,10 @@ struct Work {
   int* hk = nullptr;  // pinned host mirrors
   double* hdinfo = nullptr;
   uint32_t* herrw = nullptr;
+  double* hS = nullptr;  // the window's spectrum
+  size_t hS_n = 0;
 };
+constexpr size_t kLaneInfo = 64;  // dk (16 bytes), ddinfo (32), errw (16): one block, one copy
 
 struct tt_fit {
   // configuration
@@ -530,24 +533,24 @@ void init_lane(tt_fit* h, Work& w, cudaStream_t st, bool own_stream) {
   w.st = st;
   w.own_stream = own_stream;
   w.dnorm = h->pool.alloc<double>(1);
-  w.dk = h->pool.alloc<int>(4);
-  w.ddinfo = h->pool.alloc<double>(4);
-  w.errw = h->pool.alloc<uint32_t>(4);  // [0] error bits, [1] max Jacobi sweeps (diagnostic)
+  double* info = h->pool.alloc<double>(kLaneInfo / sizeof(double));
+  w.dk = (int*)info;                    // [0] kept rank, [1], [2] scratch exponents
+  w.ddinfo = info + 2;
+  w.errw = (uint32_t*)(info + 6);       // [0] error bits, [1] max Jacobi sweeps (diagnostic)
   CK(cudaMemsetAsync(w.errw, 0, 4 * sizeof(uint32_t), w.st));
   for (auto& e : w.ev) CK(cudaEventCreate(&e));
-  CK(cudaMallocHost(&w.hk, sizeof(int) * 4));
-  CK(cudaMallocHost(&w.hdinfo, sizeof(double) * 4));
-  CK(cudaMallocHost(&w.herrw, sizeof(uint32_t) * 4));
-  *w.herrw = 0;
+  CK(cudaMallocHost(&w.hk, kLaneInfo));  // mirrors the device block
+  w.hdinfo = (double*)w.hk + 2;
+  w.herrw = (uint32_t*)((double*)w.hk + 6);
+  memset(w.hk, 0, kLaneInfo);
 }
 
 void free_lane(Work& w) {
   if (w.st) cudaStreamSynchronize(w.st);
   for (auto& e : w.ev)
     if (e) cudaEventDestroy(e), e = nullptr;
-  if (w.hk) cudaFreeHost(w.hk), w.hk = nullptr;
-  if (w.hdinfo) cudaFreeHost(w.hdinfo), w.hdinfo = nullptr;
-  if (w.herrw) cudaFreeHost(w.herrw), w.herrw = nullptr;
+  if (w.hk) cudaFreeHost(w.hk), w.hk = nullptr, w.hdinfo = nullptr, w.herrw = nullptr;
+  if (w.hS) cudaFreeHost(w.hS), w.hS = nullptr, w.hS_n = 0;
   if (w.own_stream && w.st) cudaStreamDestroy(w.st);
   w.st = nullptr;
 }
@@ -890,9 +893,7 @@ int factorize_body(tt_fit* h, int m, int n, int sweep, int site1, int need) {
   // Theta (T, row-major) -> F copy scaled by 2^-e (e: exponent of max |Theta|, in dk[1]) so that its
   // squares stay inside the range of F; norm (flags NaN/Inf)
   int* ex = W(h).dk + 1;
-  CK(absmax_exponent<T>((const T*)W(h).Th, (long long)m * n, ex, W(h).st));
-  CK(copy_pow2<T, F>((long long)m * n, (const T*)W(h).Th, MF, ex, W(h).st));
-  CK(frob_norm<F>(MF, (long long)m * n, W(h).dnorm, W(h).errw, W(h).st));
+  CK(scale_norm<T, F>((const T*)W(h).Th, (long long)m * n, MF, ex, W(h).dnorm, W(h).errw, W(h).st));
   const int ks = h->chi_max + h->oversample;
   if (h->update == TT_UPDATE_2SITE_RSVD && ks < std::min(m, n)) {
     if constexpr (std::is_same<T, df32>::value && std::is_same<F, float>::value) {
@@ -995,13 +996,23 @@ int factorize_body(tt_fit* h, int m, int n, int sweep, int site1, int need) {
   return p;
 }
 
-// The factorisation of Theta: that of 2^-e Theta, with the singular values and
-// ||Theta|| scaled back (the singular vectors do not change).
+// The factorisation of 2^-e Theta and the truncation rule, which first scales the singular values and ||Theta||
+// back (the singular vectors do not change).
 template <typename T, typename F>
-int factorize(tt_fit* h, int m, int n, int sweep, int site1, int need = 3) {
+int factorize(tt_fit* h, int m, int n, int sweep, int site1, double tau_over_L, int chi_max, int need = 3) {
+  Work& w = W(h);
   const int p = factorize_body<T, F>(h, m, n, sweep, site1, need);
-  CK(unscale_pow2<F>(p, (F*)W(h).fS, W(h).dnorm, W(h).dk + 1, W(h).st));
+  const int cap = chi_max > 0 ? chi_max : p;
+  CK(truncate_rule<F>((F*)w.fS, p, w.dnorm, w.dk + 1, tau_over_L, cap, h->cutoff, w.dk, w.ddinfo, w.st));
   return p;
+}
+
+// Kept rank, kept and discarded weight, error word and the spectrum (p values of `bytes` each) to the host: one wait.
+void fetch_window(tt_fit* h, int p, size_t bytes) {
+  Work& w = W(h);
+  CK(cudaMemcpyAsync(w.hk, w.dk, kLaneInfo, cudaMemcpyDeviceToHost, w.st));
+  CK(cudaMemcpyAsync(w.hS, w.fS, bytes * p, cudaMemcpyDeviceToHost, w.st));
+  CK(cudaStreamSynchronize(w.st));
 }
 
 // ---------------------------------------------------------------------------
@@ -1176,19 +1187,14 @@ struct Sweeper {
       // a forward step of the site gauge keeps only U (C_l = U, C_{l+1} = U^T Theta); a boundary
       // update also needs V, the basis of the right neighbour's environment
       const bool left_only = h->gauge != TT_GAUGE_INVERSE_CANONICAL && fwd && !boundary;
-      p = factorize<T, float>(h, m, n, sweep, l + 1, left_only ? 1 : 3);
-      CK(truncate_rule<float>((const float*)W(h).fS, p, W(h).dnorm, h->tol / L, h->chi_max, h->cutoff, W(h).dk, W(h).ddinfo,
-                              W(h).st));
+      p = factorize<T, float>(h, m, n, sweep, l + 1, h->tol / L, h->chi_max, left_only ? 1 : 3);
     } else {
       using FX = typename FactT<T>::type;
-      p = factorize<T, FX>(h, m, n, sweep, l + 1);
-      CK(truncate_rule<FX>((const FX*)W(h).fS, p, W(h).dnorm, h->tol / L, h->chi_max, h->cutoff, W(h).dk, W(h).ddinfo, W(h).st));
+      p = factorize<T, FX>(h, m, n, sweep, l + 1, h->tol / L, h->chi_max);
     }
     CK(cudaEventRecord(W(h).ev[4], W(h).st));
-    CK(cudaMemcpyAsync(W(h).hk, W(h).dk, sizeof(int), cudaMemcpyDeviceToHost, W(h).st));
-    CK(cudaMemcpyAsync(W(h).hdinfo, W(h).ddinfo, 2 * sizeof(double), cudaMemcpyDeviceToHost, W(h).st));
-    CK(cudaMemcpyAsync(W(h).herrw, W(h).errw, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, W(h).st));
-    CK(cudaStreamSynchronize(W(h).st));
+    const size_t sbytes = h->fact_f32 ? sizeof(float) : sizeof(double);
+    fetch_window(h, p, sbytes);
     if (*W(h).herrw & ERRW_HPFAIL) {
       // the FP64-class sketch basis could not be formed (a rank-deficient sketch): clear the
       // flag and factorise this window again with the all-FP32 randomized update
@@ -1196,19 +1202,14 @@ struct Sweeper {
       W(h).hp_off = true;
       const bool left_only = h->gauge != TT_GAUGE_INVERSE_CANONICAL && fwd && !boundary;
       try {
-        p = factorize<T, float>(h, m, n, sweep, l + 1, left_only ? 1 : 3);
+        p = factorize<T, float>(h, m, n, sweep, l + 1, h->tol / L, h->chi_max, left_only ? 1 : 3);
       } catch (...) {
         W(h).hp_off = false;
         throw;
       }
       W(h).hp_off = false;
-      CK(truncate_rule<float>((const float*)W(h).fS, p, W(h).dnorm, h->tol / L, h->chi_max, h->cutoff, W(h).dk,
-                              W(h).ddinfo, W(h).st));
       CK(cudaEventRecord(W(h).ev[4], W(h).st));
-      CK(cudaMemcpyAsync(W(h).hk, W(h).dk, sizeof(int), cudaMemcpyDeviceToHost, W(h).st));
-      CK(cudaMemcpyAsync(W(h).hdinfo, W(h).ddinfo, 2 * sizeof(double), cudaMemcpyDeviceToHost, W(h).st));
-      CK(cudaMemcpyAsync(W(h).herrw, W(h).errw, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, W(h).st));
-      CK(cudaStreamSynchronize(W(h).st));
+      fetch_window(h, p, sbytes);
       ++W(h).hp_fallbacks;
     }
     add(2, 0, 1);
@@ -1255,16 +1256,9 @@ struct Sweeper {
       CK(cudaEventRecord(W(h).ev[9], W(h).st));
       W(h).connect_pending = true;
     }
-    // host copy of the kept spectrum for tt_fit_result
-    if (h->fact_f32) {
-      std::vector<float> sv(k);
-      CK(cudaMemcpyAsync(sv.data(), W(h).fS, sizeof(float) * k, cudaMemcpyDeviceToHost, W(h).st));
-      h->lam[l + 1].assign(sv.begin(), sv.end());
-    } else {
-      std::vector<double> sv(k);
-      CK(cudaMemcpyAsync(sv.data(), W(h).fS, sizeof(double) * k, cudaMemcpyDeviceToHost, W(h).st));
-      h->lam[l + 1].assign(sv.begin(), sv.end());
-    }
+    // host copy of the kept spectrum for tt_fit_result (fetched with the rank: a copy here would wait for the update)
+    if (h->fact_f32) h->lam[l + 1].assign((const float*)W(h).hS, (const float*)W(h).hS + k);
+    else h->lam[l + 1].assign((const double*)W(h).hS, (const double*)W(h).hS + k);
   }
 
   void run(int n_sweeps) {
@@ -1458,6 +1452,12 @@ void allocate_chain(tt_fit* h) {
                        &w.fR2, &w.pU, &w.pV, &w.pG, &w.pT})
       *f = calloc_chain<double>(h, w.fsz);
     w.fS = calloc_chain<double>(h, side);
+    if (w.hS_n < (size_t)side) {
+      if (w.hS) cudaFreeHost(w.hS);
+      w.hS = nullptr;
+      CK(cudaMallocHost(&w.hS, sizeof(double) * side));
+      w.hS_n = side;
+    }
     w.pP = calloc_chain<double>(h, (size_t)side * ks + (size_t)ks * ks + 64);
     if (std::is_same<T, df32>::value) {  // the tensor-core GEMM of the DF32 chain
       w.oz_slice = (size_t)OZ_DIGITS * 2 * omax;
@@ -1736,8 +1736,7 @@ void vidal_init(tt_fit* h) {
       const int m = D.c[j] * D.ds[j] * D.dt[j], n = D.c[j + 1];
       copymap<double, T>(h, m, n, h->C64[j], IdxMap::lin(n), IdxMap::lin(1), (T*)W(h).Th, IdxMap::lin(n),
                          IdxMap::lin(1));
-      const int p = factorize<T, F>(h, m, n, 0, j + 1);
-      CK(truncate_rule<F>((const F*)W(h).fS, p, W(h).dnorm, 0.0, p, h->cutoff, W(h).dk, W(h).ddinfo, W(h).st));
+      const int p = factorize<T, F>(h, m, n, 0, j + 1, 0.0, 0);
       CK(cudaMemcpyAsync(W(h).hk, W(h).dk, sizeof(int), cudaMemcpyDeviceToHost, W(h).st));
       CK(cudaMemcpyAsync(W(h).herrw, W(h).errw, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, W(h).st));
       CK(cudaStreamSynchronize(W(h).st));
@@ -2250,7 +2249,7 @@ void zipup_rl(tt_fit* h, const ZipArgs& z, std::vector<double*>& C, std::vector<
       zgemm<T>(h, g, ws, wse, false);
     }
     CK(fix_signs<T>((int)n, 0, pv, Vn, (int)n, nullptr, 0, st));
-    CK(truncate_rule<T>(Sv, pv, w.dnorm, z.tol / L, z.chi_max, z.cutoff, w.dk, w.ddinfo, st));
+    CK(truncate_rule<T>(Sv, pv, w.dnorm, nullptr, z.tol / L, z.chi_max, z.cutoff, w.dk, w.ddinfo, st));
     CK(cudaMemcpyAsync(w.hk, w.dk, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(w.herrw, w.errw, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));

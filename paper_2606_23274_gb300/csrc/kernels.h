@@ -114,8 +114,9 @@ cudaError_t frob_norm(const T* x, long long n, double* out, uint32_t* errw, cuda
 
 // Truncation rule (Sec. 2.3.4): from sorted S (p values), ||M||_F, writes
 // info[0] = k, and dinfo[0] = sum_{j<k} s_j^2, dinfo[1] = sqrt(sum_{j>=k} s_j^2)/||M||_F.
+// With e (device): S and ||M|| are those of 2^-e M and are scaled back first, in place.
 template <typename F>
-cudaError_t truncate_rule(const F* S, int p, const double* normM, double tau_over_L, int chi_max,
+cudaError_t truncate_rule(F* S, int p, double* normM, const int* e, double tau_over_L, int chi_max,
                           double cutoff, int* info, double* dinfo, cudaStream_t st);
 
 // x_j = sqrt(max(x_j, 0)) (singular values from Gram eigenvalues)
@@ -153,8 +154,9 @@ template <typename T>
 cudaError_t absmax_exponent(const T* x, long long n, int* e, cudaStream_t st);
 template <typename Tin, typename Tout>
 cudaError_t copy_pow2(long long n, const Tin* in, Tout* out, const int* e, cudaStream_t st);
-template <typename F>
-cudaError_t unscale_pow2(int p, F* s, double* nrm, const int* e, cudaStream_t st);
+// out = 2^-e x with e the exponent of max |x| (written to *e), *nrm = ||out||_F; flags non-finite values
+template <typename T, typename F>
+cudaError_t scale_norm(const T* x, long long n, F* out, int* e, double* nrm, uint32_t* errw, cudaStream_t st);
 // out (cols x rows) = (in diag(y))^T in type T
 template <typename T>
 cudaError_t scale_cols_t(int rows, int cols, const double* in, const double* y, T* out, cudaStream_t st);

@@ -1325,11 +1325,18 @@ __device__ __forceinline__ double suffix_from(double v, int lane) {  // sum over
   return v;
 }
 template <typename F>
-__global__ void truncate_kernel(const F* S, int p, const double* normM, double tau_over_L, int chi_max,
+__global__ void truncate_kernel(F* S, int p, double* normM, const int* e, double tau_over_L, int chi_max,
                                 double cutoff, int* info, double* dinfo) {
   const int lane = threadIdx.x;
   const int run = (p + 31) / 32, j0 = min(p, lane * run), j1 = min(p, j0 + run);
-  const double nM = *normM;
+  double nM = *normM;
+  if (e) {  // the decomposition was that of 2^-e M: s_j <- s_j 2^e, ||M|| <- ||M|| 2^e
+    const int ex = *e;
+    for (int j = j0; j < j1; ++j) S[j] = (F)scalbn((double)S[j], ex);
+    nM = scalbn(nM, ex);
+    __syncwarp();
+    if (lane == 0) *normM = nM;
+  }
   double sq = 0.0;  // of my run
   for (int j = j1 - 1; j >= j0; --j) sq += (double)S[j] * (double)S[j];
   int k = min(chi_max, p);
@@ -1370,15 +1377,15 @@ __global__ void truncate_kernel(const F* S, int p, const double* normM, double t
 }
 
 template <typename F>
-cudaError_t truncate_rule(const F* S, int p, const double* normM, double tau_over_L, int chi_max, double cutoff,
+cudaError_t truncate_rule(F* S, int p, double* normM, const int* e, double tau_over_L, int chi_max, double cutoff,
                           int* info, double* dinfo, cudaStream_t st) {
   ++tl_launches;
-  truncate_kernel<F><<<1, 32, 0, st>>>(S, p, normM, tau_over_L, chi_max, cutoff, info, dinfo);
+  truncate_kernel<F><<<1, 32, 0, st>>>(S, p, normM, e, tau_over_L, chi_max, cutoff, info, dinfo);
   return cudaGetLastError();
 }
-template cudaError_t truncate_rule<double>(const double*, int, const double*, double, int, double, int*, double*,
+template cudaError_t truncate_rule<double>(double*, int, double*, const int*, double, int, double, int*, double*,
                                            cudaStream_t);
-template cudaError_t truncate_rule<float>(const float*, int, const double*, double, int, double, int*, double*,
+template cudaError_t truncate_rule<float>(float*, int, double*, const int*, double, int, double, int*, double*,
                                           cudaStream_t);
 
 // s_j = sqrt(max(lambda_j, 0)): singular values from the eigenvalues of a Gram matrix
@@ -1842,21 +1849,77 @@ template cudaError_t copy_pow2<float, float>(long long, const float*, float*, co
 template cudaError_t copy_pow2<df32, float>(long long, const df32*, float*, const int*, cudaStream_t);
 template cudaError_t copy_pow2<df32, double>(long long, const df32*, double*, const int*, cudaStream_t);
 
-// s_i <- s_i 2^e and ||M|| <- ||M|| 2^e: the factorisation of 2^-e M back to M
-template <typename F>
-__global__ void unscale_pow2_kernel(int p, F* s, double* nrm, const int* e) {
-  const int ex = *e;
-  for (int i = threadIdx.x; i < p; i += blockDim.x) s[i] = (F)scalbn((double)s[i], ex);
-  if (threadIdx.x == 0) *nrm = scalbn(*nrm, ex);
+// 2^-e x in type F and its norm in one launch: one cluster of up to 8 CTAs takes the largest exponent e, then
+// scales, stores and sums (three launches and a memset before; the second read comes from L2). Everything as
+// absmax_exponent, copy_pow2 and frob_norm one after the other give it.
+template <typename T, typename F>
+__global__ void __launch_bounds__(1024) scale_norm_kernel(const T* __restrict__ x, long long n, F* __restrict__ out,
+                                                          int* e, double* nrm, uint32_t* errw) {
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ double red[32];
+  __shared__ double total[8];
+  __shared__ int mine, top[8];
+  const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  if (threadIdx.x == 0) mine = (int)0x80808080;
+  __syncthreads();
+  int m = INT_MIN;
+#pragma unroll 4
+  for (long long i = i0; i < n; i += step) {
+    const T v = x[i];
+    if (!is_zero(v)) m = max(m, exp_of(v));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m != INT_MIN) atomicMax(&mine, m);
+  __syncthreads();
+  if (threadIdx.x < gridDim.x) *cl.map_shared_rank(&top[blockIdx.x], threadIdx.x) = mine;
+  cl.sync();
+  int ex = top[0];
+  for (unsigned c = 1; c < gridDim.x; ++c) ex = max(ex, top[c]);
+  F part = 0;
+  bool bad = false;
+#pragma unroll 4
+  for (long long i = i0; i < n; i += step) {
+    const F v = scale_pow2<F, T>(x[i], -ex);
+    out[i] = v;
+    bad |= !isfinite(v);
+    part += v * v;
+  }
+  const double s = block_sum((double)part, red);
+  bad = __syncthreads_or(bad);
+  if (threadIdx.x == 0) {
+    *cl.map_shared_rank(&total[blockIdx.x], 0) = s;
+    if (bad && errw) atomicOr(errw, ERRW_NAN);
+  }
+  cl.sync();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double t = 0;
+    for (unsigned c = 0; c < gridDim.x; ++c) t += total[c];
+    *nrm = sqrt(t);
+    *e = ex;
+  }
 }
-template <typename F>
-cudaError_t unscale_pow2(int p, F* s, double* nrm, const int* e, cudaStream_t st) {
+template <typename T, typename F>
+cudaError_t scale_norm(const T* x, long long n, F* out, int* e, double* nrm, uint32_t* errw, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n <= 8192 ? 1 : 8);  // one cluster
+  cfg.blockDim = dim3(1024);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cfg.gridDim.x;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   ++tl_launches;
-  unscale_pow2_kernel<F><<<1, 256, 0, st>>>(p, s, nrm, e);
-  return cudaGetLastError();
+  cudaError_t r = cudaLaunchKernelEx(&cfg, scale_norm_kernel<T, F>, x, n, out, e, nrm, errw);
+  return r != cudaSuccess ? r : cudaGetLastError();
 }
-template cudaError_t unscale_pow2<float>(int, float*, double*, const int*, cudaStream_t);
-template cudaError_t unscale_pow2<double>(int, double*, double*, const int*, cudaStream_t);
+template cudaError_t scale_norm<double, double>(const double*, long long, double*, int*, double*, uint32_t*, cudaStream_t);
+template cudaError_t scale_norm<double, float>(const double*, long long, float*, int*, double*, uint32_t*, cudaStream_t);
+template cudaError_t scale_norm<float, float>(const float*, long long, float*, int*, double*, uint32_t*, cudaStream_t);
+template cudaError_t scale_norm<df32, float>(const df32*, long long, float*, int*, double*, uint32_t*, cudaStream_t);
+template cudaError_t scale_norm<df32, double>(const df32*, long long, double*, int*, double*, uint32_t*, cudaStream_t);
 }  // namespace ttfit
 
 namespace ttfit {

@@ -70,7 +70,7 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   if ((e = fix_signs<double>(tr ? r : q, tr ? q : r, r, tr ? Vx : Ux, tr ? r : q, tr ? Ux : Vx, tr ? q : r, st)) !=
       cudaSuccess)
     return e;
-  if ((e = truncate_rule<double>(Sv, r, nrm, tau_rel, chi_max, 1e-13, k_dev, dinfo, st)) != cudaSuccess) return e;
+  if ((e = truncate_rule<double>(Sv, r, nrm, nullptr, tau_rel, chi_max, 1e-13, k_dev, dinfo, st)) != cudaSuccess) return e;
   const long long tot = (long long)q * r;
   const int blocks = (int)std::max<long long>(1, std::min<long long>((tot + 255) / 256, 1024));
   ++tl_launches;
