@@ -931,15 +931,14 @@ int factorize_body(tt_fit* h, int m, int n, int sweep, int site1, int need) {
       CK(fix_signs<F>(m, n, ks, fUM, m, (F*)nullptr, n, W(h).st));
       return ks;
     }
-    if constexpr (std::is_same<F, double>::value) {
-      // on R2^T, whose columns are graded (see svd_tall64): R2^T = Vr S Ur^T
-      copymap<F, F>(h, ks, ks, fR2, IdxMap::lin(1), IdxMap::lin(ks), fX, IdxMap::lin(ks), IdxMap::lin(1));
-      const cudaError_t e = svd_graded64(ks, fX, fV, fS, fU, fBt, fOm, 60, W(h).errw, h->sm_count, W(h).st);
-      if (e == cudaErrorNotSupported) jac(ks, ks, fX, fV, fS, fU);
-      else CK(e);
-    } else {
-      jac(ks, ks, fR2, fU, fS, fV);               // R2 = Ur S Vr^T
-    }
+    // on R2^T, whose columns are graded (see svd_graded64): R2^T = Vr S Ur^T. On R2 itself Jacobi takes twice the sweeps,
+    // and here Ur, the basis of a backward step, is the product of the rotations, orthonormal to rounding
+    copymap<F, F>(h, ks, ks, fR2, IdxMap::lin(1), IdxMap::lin(ks), fX, IdxMap::lin(ks), IdxMap::lin(1));
+    cudaError_t e = cudaErrorNotSupported;
+    if constexpr (std::is_same<F, double>::value)
+      e = svd_graded64(ks, fX, fV, fS, fU, fBt, fOm, 60, W(h).errw, h->sm_count, W(h).st);
+    if (e == cudaErrorNotSupported) jac(ks, ks, fX, fV, fS, fU);
+    else CK(e);
     GemmArgs<F> g3;  // U_M = Q Vr (m x ks)
     g3.M = m; g3.N = ks; g3.K = ks;
     g3.A = fQ; g3.am = IdxMap::lin(1); g3.ak = IdxMap::lin(m); g3.a_kfast = false;
