@@ -18,7 +18,9 @@ namespace {
 // the rows allow it) and walks down the rows: the column's split into (j_a, j_b) is done once, and the entries
 // of A and B come from L1. Narrow sites put several rows side by side in a block. All sites of a call go into
 // one launch, so that short sites do not each leave a last wave and a gap behind.
-// L = 8, chi 48 x 40, FP32 (354 MB): one thread an element with 64-bit divisions took 748 us.
+// L = 8, chi 48 x 40, FP32 (354 MB, a call): one thread an element with 64-bit divisions took 748 us; so, with
+// scalar loads of A and B for every column 218, with vector loads of B 156 (C at 2.3 TB/s, the host's part of the
+// call included).
 constexpr int NP_SITES = 32;  // sites of one launch (the table is a kernel parameter)
 constexpr int NP_ROWS = 16;   // rows a thread walks down
 
@@ -29,7 +31,7 @@ struct NaiveSite {
   int a0, a1, b0, b1, s, u, t;
   int cx;      // threads along the columns (a power of two <= 256), 256 / cx rows side by side
   long long ncol;  // column tiles
-  int vec;     // 16-byte stores
+  int vec;     // 1: 16-byte stores, 2: 16-byte loads of B as well
   long long first;  // first block of the site
 };
 template <typename F>
@@ -38,7 +40,8 @@ struct NaiveTable {
   int n;
 };
 
-template <typename F, int VW>
+// BLOCK: b1 is a multiple of VW, so that the VW columns share j_a and their entries of B are one aligned vector.
+template <typename F, int VW, bool BLOCK>
 __device__ __forceinline__ void naive_tile(const NaiveSite<F>& S, long long tile) {
   const int cx = S.cx, ry = 256 / cx;
   const long long cols = (long long)S.a1 * S.b1, ct = tile % S.ncol, rt = tile / S.ncol;
@@ -69,8 +72,18 @@ __device__ __forceinline__ void naive_tile(const NaiveSite<F>& S, long long tile
 #pragma unroll
     for (int v = 0; v < VW; ++v) acc[v] = F(0);
     for (int uu = 0; uu < S.u; ++uu) {
+      if constexpr (BLOCK) {
+        struct __align__(16) V {
+          F e[VW];
+        };
+        const F x = pa[ja[0]];
+        const V y = *reinterpret_cast<const V*>(pb + jb[0]);
 #pragma unroll
-      for (int v = 0; v < VW; ++v) acc[v] += pa[ja[v]] * pb[jb[v]];
+        for (int v = 0; v < VW; ++v) acc[v] += x * y.e[v];
+      } else {
+#pragma unroll
+        for (int v = 0; v < VW; ++v) acc[v] += pa[ja[v]] * pb[jb[v]];
+      }
       pa += S.a1;
       pb += (long long)S.t * S.b1;
     }
@@ -86,8 +99,9 @@ __global__ void __launch_bounds__(256) naive_product_kernel(const __grid_constan
   int k = 0;
   while (k + 1 < T.n && (long long)blockIdx.x >= T.site[k + 1].first) ++k;
   const NaiveSite<F>& S = T.site[k];
-  if (S.vec) naive_tile<F, 16 / (int)sizeof(F)>(S, blockIdx.x - S.first);
-  else naive_tile<F, 1>(S, blockIdx.x - S.first);
+  if (S.vec == 2) naive_tile<F, 16 / (int)sizeof(F), true>(S, blockIdx.x - S.first);
+  else if (S.vec) naive_tile<F, 16 / (int)sizeof(F), false>(S, blockIdx.x - S.first);
+  else naive_tile<F, 1, false>(S, blockIdx.x - S.first);
 }
 
 template <typename F>
@@ -106,7 +120,8 @@ cudaError_t naive_product(const tt_mpo_desc* A, const tt_mpo_desc* B, const tt_m
       S.a0 = A->bond[l], S.a1 = A->bond[l + 1], S.b0 = B->bond[l], S.b1 = B->bond[l + 1];
       S.s = A->d_out[l], S.u = A->d_in[l], S.t = B->d_in[l];
       const long long cols = (long long)S.a1 * S.b1, rows = (long long)S.a0 * S.b0 * S.s * S.t;
-      S.vec = cols % VW == 0 && ((uintptr_t)S.C & 15) == 0;
+      S.vec = cols % VW == 0 && ((uintptr_t)S.C & 15) == 0 ? 1 : 0;
+      if (S.vec && S.b1 % VW == 0 && ((uintptr_t)S.B & 15) == 0) S.vec = 2;  // a row's entries of B are aligned too
       const long long wide = S.vec ? cols / VW : cols;
       S.cx = 1;
       while (S.cx < 256 && S.cx < wide) S.cx *= 2;
