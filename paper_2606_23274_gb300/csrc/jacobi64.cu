@@ -388,7 +388,8 @@ cudaError_t jacobi_svd64(int q, int p, const double* W, const double* Vin, doubl
 // stopping rule instead of 10 (spectra down to 1e-18 s_1: the columns are graded, so FP32 keeps each to its own
 // rounding). The result is as accurate as without: every rotation that counts is taken in FP64.
 // U must not be L; e0, e1: p x p scratch each, or null (no room: all sweeps in FP64).
-// 128 x 128: 3.3 ms by FP64 sweeps alone.
+// 128 x 128 in an FP64 fit: 3.3 ms by FP64 sweeps alone; so 0.6 ms of FP32 sweeps, 0.9 ms of FP64 ones and six
+// products of 10 us. 256 x 256: 13 ms; 1.9, 4.0 and 0.3.
 cudaError_t svd_graded64(int p, const double* L, double* U, double* Sv, double* W, double* e0, double* e1, int max_sweeps,
                          uint32_t* errw, int sm_count, cudaStream_t st) {
   Jacobi64Plan plan;
