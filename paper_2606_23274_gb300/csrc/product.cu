@@ -19,8 +19,8 @@ namespace {
 // of A and B come from L1. Narrow sites put several rows side by side in a block. All sites of a call go into
 // one launch, so that short sites do not each leave a last wave and a gap behind.
 // L = 8, chi 48 x 40, FP32 (354 MB, a call): one thread an element with 64-bit divisions took 748 us; so, with
-// scalar loads of A and B for every column 218, with vector loads of B 156 (C at 2.3 TB/s, the host's part of the
-// call included).
+// scalar loads of A and B for every column 218, with vector loads of B 156, and with each row's digits stepped on
+// from the last row's, where four divisions a row were most of the instructions, 120 (C at 2.9 TB/s).
 constexpr int NP_SITES = 32;  // sites of one launch (the table is a kernel parameter)
 constexpr int NP_ROWS = 16;   // rows a thread walks down
 
@@ -52,20 +52,29 @@ __device__ __forceinline__ void naive_tile(const NaiveSite<F>& S, long long tile
   for (int v = 0; v < VW; ++v) ja[v] = (int)((col + v) / S.b1), jb[v] = (int)((col + v) - (long long)ja[v] * S.b1);
   const long long rows = (long long)S.a0 * S.b0 * S.s * S.t;
   long long row = rt * (NP_ROWS * ry) + threadIdx.x / cx;
+  // the row's digits (i_a, i_b, s, t) come from divisions once; then the digits of ry are added with their carries
+  unsigned tt, ss, ib, ia, dt = ry, ds, db, da;
+  if (rows <= 0x7FFFFFFF) {
+    unsigned r = (unsigned)row;
+    tt = r % (unsigned)S.t, r /= (unsigned)S.t;
+    ss = r % (unsigned)S.s, r /= (unsigned)S.s;
+    ib = r % (unsigned)S.b0, ia = r / (unsigned)S.b0;
+  } else {
+    long long r = row;
+    tt = (unsigned)(r % S.t), r /= S.t;
+    ss = (unsigned)(r % S.s), r /= S.s;
+    ib = (unsigned)(r % S.b0), ia = (unsigned)(r / S.b0);
+  }
+  ds = dt / (unsigned)S.t, dt %= (unsigned)S.t;
+  db = ds / (unsigned)S.s, ds %= (unsigned)S.s;
+  da = db / (unsigned)S.b0, db %= (unsigned)S.b0;
+  auto carry = [](unsigned& x, unsigned n) {  // x < 2n on entry (n < 2^31)
+    const unsigned c = x >= n;
+    x -= c ? n : 0u;
+    return c;
+  };
 #pragma unroll 2
   for (int i = 0; i < NP_ROWS && row < rows; ++i, row += ry) {
-    int tt, ss, ib, ia;
-    if (rows <= 0x7FFFFFFF) {
-      unsigned r = (unsigned)row;
-      tt = (int)(r % (unsigned)S.t), r /= (unsigned)S.t;
-      ss = (int)(r % (unsigned)S.s), r /= (unsigned)S.s;
-      ib = (int)(r % (unsigned)S.b0), ia = (int)(r / (unsigned)S.b0);
-    } else {
-      long long r = row;
-      tt = (int)(r % S.t), r /= S.t;
-      ss = (int)(r % S.s), r /= S.s;
-      ib = (int)(r % S.b0), ia = (int)(r / S.b0);
-    }
     const F* pa = S.A + ((long long)ia * S.s + ss) * S.u * S.a1;
     const F* pb = S.B + ((long long)ib * S.u * S.t + tt) * S.b1;
     F acc[VW];
@@ -91,6 +100,10 @@ __device__ __forceinline__ void naive_tile(const NaiveSite<F>& S, long long tile
     if constexpr (VW == 1) out[0] = acc[0];
     else if constexpr (VW == 2) *reinterpret_cast<double2*>(out) = make_double2(acc[0], acc[1]);
     else *reinterpret_cast<float4*>(out) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    tt += dt;
+    ss += ds + carry(tt, (unsigned)S.t);
+    ib += db + carry(ss, (unsigned)S.s);
+    ia += da + carry(ib, (unsigned)S.b0);
   }
 }
 
