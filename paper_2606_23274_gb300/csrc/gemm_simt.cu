@@ -247,37 +247,49 @@ __global__ void __launch_bounds__(128) gemm_f32_kernel(GemmArgs<float> g, float*
   }
 }
 
-// Sum of the split-K partials into the output layouts. A block takes 8 rows of 32 columns: the partials are read
+// Sum of the split-K partials into the output layouts. A block takes R rows of 32 columns: the partials are read
 // along the columns, each output is written along its own fast direction, and the index maps are evaluated once
 // a row and column of the tile (four maps and a 64-bit division an element took 20 us for 512 x 512 df32).
-template <typename T>
+// R = 32 keeps four loads a thread in flight where one partial is all there is (32768 x 256 df32, the digit
+// products: 66 us with 8 rows, 51 so); R = 8 spreads small outputs over the SMs (512 x 512, 32 partials: 11.7 us).
+template <typename T, int R>
 __global__ void __launch_bounds__(256) splitk_reduce_kernel(GemmArgs<T> g, const T* __restrict__ ws, int splits) {
-  __shared__ T tile[8][33];
-  __shared__ long long rm[8], rm2[8], cn[32], cn2[32];
+  __shared__ T tile[R][33];
+  __shared__ long long rm[R], rm2[R], cn[32], cn2[32];
   const int t = threadIdx.x;
   const long long total = (long long)g.M * g.N;
-  const int nct = (g.N + 31) / 32, nrt = (g.M + 7) / 8;
+  const int nct = (g.N + 31) / 32, nrt = (g.M + R - 1) / R;
   for (long long b = blockIdx.x; b < (long long)nct * nrt; b += gridDim.x) {
-    const int m0 = (int)(b / nct) * 8, n0 = (int)(b % nct) * 32;
+    const int m0 = (int)(b / nct) * R, n0 = (int)(b % nct) * 32;
     if (t < 32) cn[t] = g.cn(min(n0 + t, g.N - 1));
-    else if (t < 40) rm[t - 32] = g.cm(min(m0 + t - 32, g.M - 1));
+    else if (t < 32 + R) rm[t - 32] = g.cm(min(m0 + t - 32, g.M - 1));
     else if (g.C2 && t >= 64 && t < 96) cn2[t - 64] = g.cn2(min(n0 + t - 64, g.N - 1));
-    else if (g.C2 && t >= 96 && t < 104) rm2[t - 96] = g.cm2(min(m0 + t - 96, g.M - 1));
+    else if (g.C2 && t >= 96 && t < 96 + R) rm2[t - 96] = g.cm2(min(m0 + t - 96, g.M - 1));
     {
       const int i = t >> 5, j = t & 31;
-      T s = T(0);
-      if (m0 + i < g.M && n0 + j < g.N) {
-        const T* w = ws + (size_t)(m0 + i) * g.N + n0 + j;
-#pragma unroll 4
-        for (int z = 0; z < splits; ++z) s += w[(size_t)z * total];
-        s = g.alpha * s;
+      T s[R / 8];
+      const T* w[R / 8];  // rows past the end read the last one, so that no test stands between the loads
+#pragma unroll
+      for (int k = 0; k < R / 8; ++k) {
+        s[k] = T(0);
+        w[k] = ws + (size_t)min(m0 + i + 8 * k, g.M - 1) * g.N + n0 + j;
       }
-      tile[i][j] = s;
+      if (n0 + j < g.N) {
+#pragma unroll 4
+        for (int z = 0; z < splits; ++z)
+#pragma unroll
+          for (int k = 0; k < R / 8; ++k) s[k] += w[k][(size_t)z * total];
+      }
+#pragma unroll
+      for (int k = 0; k < R / 8; ++k) tile[i + 8 * k][j] = g.alpha * s[k];
     }
     __syncthreads();
     auto each = [&](bool along_rows, auto put) {  // along_rows: neighbouring threads take neighbouring rows
-      const int i = along_rows ? t & 7 : t >> 5, j = along_rows ? t >> 3 : t & 31;
-      if (m0 + i < g.M && n0 + j < g.N) put(i, j);
+#pragma unroll
+      for (int k = 0; k < R / 8; ++k) {
+        const int i = along_rows ? t % R : (t >> 5) + 8 * k, j = along_rows ? t / R + 256 / R * k : t & 31;
+        if (m0 + i < g.M && n0 + j < g.N) put(i, j);
+      }
     };
     if (g.C2) each(g.cn2.s2 != 1, [&](int i, int j) { g.C2[rm2[i] + cn2[j]] = tile[i][j]; });
     each(g.cn.s2 != 1, [&](int i, int j) {
@@ -292,11 +304,13 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(GemmArgs<T> g, const
 
 template <typename T>
 cudaError_t splitk_reduce(const GemmArgs<T>& g, const T* ws, int splits, int sm_count, cudaStream_t st) {
-  const long long tiles = (long long)((g.N + 31) / 32) * ((g.M + 7) / 8);
-  const int blocks = (int)(tiles < (1 << 16) ? tiles : (1 << 16));
-  (void)sm_count;
+  const long long nct = (g.N + 31) / 32, tall = nct * ((g.M + 31) / 32);
+  const bool big = tall >= 8LL * sm_count;  // the 32-row blocks fill the SMs: 2048 of them 19.3 us, with 8 rows 19.8
+  const long long tiles = big ? tall : nct * ((g.M + 7) / 8);
+  const int blocks = (int)(tiles < 1 ? 1 : tiles < (1 << 16) ? tiles : (1 << 16));
   ++tl_launches;
-  splitk_reduce_kernel<T><<<blocks < 1 ? 1 : blocks, 256, 0, st>>>(g, ws, splits);
+  if (big) splitk_reduce_kernel<T, 32><<<blocks, 256, 0, st>>>(g, ws, splits);
+  else splitk_reduce_kernel<T, 8><<<blocks, 256, 0, st>>>(g, ws, splits);
   return cudaGetLastError();
 }
 template cudaError_t splitk_reduce<double>(const GemmArgs<double>&, const double*, int, int, cudaStream_t);
@@ -310,7 +324,7 @@ cudaError_t gemm_simt(const GemmArgs<T>& g, T* ws, size_t ws_elems, int sm_count
     GemmArgs<T> z = g;
     z.alpha = T(0);
     ++tl_launches;
-    splitk_reduce_kernel<T><<<256, 256, 0, st>>>(z, nullptr, 0);
+    splitk_reduce_kernel<T, 8><<<256, 256, 0, st>>>(z, nullptr, 0);
     return cudaGetLastError();
   }
   const bool slow = std::is_same<T, double>::value || std::is_same<T, df32>::value;
