@@ -1268,6 +1268,7 @@ __global__ void __launch_bounds__(1024) frob_kernel(const T* __restrict__ x, lon
   // per-thread partial in the value type (FP32 stays on the FP32 pipes)
   using P = typename std::conditional<std::is_same<T, float>::value, float, double>::type;
   cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_arrive();  // waited for before the first store into another CTA: every CTA must have started
   __shared__ double red[32];
   __shared__ double total[8];
   P part = 0;
@@ -1281,6 +1282,7 @@ __global__ void __launch_bounds__(1024) frob_kernel(const T* __restrict__ x, lon
   }
   const double s = block_sum((double)part, red);
   bad = __syncthreads_or(bad);
+  cl.barrier_wait();
   if (threadIdx.x == 0) {
     *cl.map_shared_rank(&total[blockIdx.x], 0) = s;
     if (bad && errw) atomicOr(errw, ERRW_NAN);
@@ -1853,6 +1855,7 @@ template <typename T, typename F>
 __global__ void __launch_bounds__(1024) scale_norm_kernel(const T* __restrict__ x, long long n, F* __restrict__ out,
                                                           int* e, double* nrm, uint32_t* errw) {
   cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_arrive();  // as in frob_kernel
   __shared__ double red[32];
   __shared__ double total[8];
   __shared__ int mine, top[8];
@@ -1868,6 +1871,7 @@ __global__ void __launch_bounds__(1024) scale_norm_kernel(const T* __restrict__ 
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0 && m != INT_MIN) atomicMax(&mine, m);
   __syncthreads();
+  cl.barrier_wait();
   if (threadIdx.x < gridDim.x) *cl.map_shared_rank(&top[blockIdx.x], threadIdx.x) = mine;
   cl.sync();
   int ex = top[0];
