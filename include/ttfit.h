@@ -269,7 +269,8 @@ tt_status tt_fit_exec_flops(const tt_fit* h, double out[2]);
 tt_status tt_fit_launch_count(const tt_fit* h, long long* n);
 
 /* Device memory of the handles (and the scratch of tt_mpo_grad and
- * tt_svd_truncated) comes from a process-wide cache of blocks: tt_fit_destroy (and the release of buffers that a handle no longer needs)
+ * tt_svd_truncated) comes from a process-wide cache of blocks: tt_fit_destroy
+ * (and the release of buffers that a handle no longer needs)
  * returns blocks to it instead of freeing them, and later handles reuse them
  * without allocating (best fit: the smallest cached block of at least the size
  * asked for and at most twice it). At most a quarter of a device's memory (and
@@ -353,8 +354,8 @@ tt_status tt_mpo_grad(const tt_mpo_desc* A, const tt_mpo_desc* B, const tt_mpo_d
  * row-major), r = min(m, n) <= 1024, and returns in *k_out (host) the rank
  * the truncation rule keeps: k = min(chi_max, min{k : sqrt(sum_{j>k} s_j^2)
  * <= tau_rel ||M||_F}), values <= 1e-13 s_1 dropped, k >= 1. Takes its
- * scratch from the block cache (tt_device_cache_release), runs on `stream` (cudaStream_t, NULL = default)
- * and synchronises it. Errors: TT_ERR_INVALID_ARGUMENT (NULL pointer,
+ * scratch from the block cache (tt_device_cache_release), runs on `stream`
+ * (cudaStream_t, NULL = default) and synchronises it. Errors: TT_ERR_INVALID_ARGUMENT (NULL pointer,
  * non-positive size, r > 1024), TT_ERR_OUT_OF_MEMORY, TT_ERR_CUDA,
  * TT_ERR_NUMERICAL (non-finite input, no convergence). */
 tt_status tt_svd_truncated(const double* M, int m, int n, int chi_max, double tau_rel, double* U, double* S,
