@@ -11,19 +11,10 @@ namespace cg = cooperative_groups;
 
 namespace ttfit {
 
-// Arithmetic of the register QR in its three types.
+// Arithmetic of the register QR in its two types. null: the squared norm of a column without a reflector; finite: one
+// that is neither infinite (an entry, or its square) nor NaN.
 template <typename C>
 struct QrArith;
-
-template <>
-struct QrArith<float> {
-  static __device__ __forceinline__ float fma(float a, float b, float c) { return fmaf(a, b, c); }
-  static __device__ __forceinline__ float sqrt(float x) { return sqrtf(x); }
-  static __device__ __forceinline__ float rcp(float x) { return 1.0f / x; }
-  static __device__ __forceinline__ float abs(float x) { return fabsf(x); }
-  static __device__ __forceinline__ bool neg(float x) { return x < 0.0f; }
-  static __device__ __forceinline__ bool live(float ss) { return ss > 0.0f && ss < INFINITY; }
-};
 
 template <>
 struct QrArith<df32> {
@@ -32,7 +23,8 @@ struct QrArith<df32> {
   static __device__ __forceinline__ df32 rcp(df32 x) { return qrcp(x); }
   static __device__ __forceinline__ df32 abs(df32 x) { return x.hi < 0.0f ? -x : x; }
   static __device__ __forceinline__ bool neg(df32 x) { return x.hi < 0.0f; }
-  static __device__ __forceinline__ bool live(df32 ss) { return ss.hi > 0.0f && ss.hi < INFINITY; }
+  static __device__ __forceinline__ bool null(df32 ss) { return ss.hi <= 0.0f; }
+  static __device__ __forceinline__ bool finite(df32 ss) { return isfinite(ss.hi); }
 };
 
 // FP64: the FP64 pipe takes 64 cycles for a warp instruction on this GPU, so square root and reciprocal
@@ -77,9 +69,8 @@ struct QrArith<double> {
     return __hiloint2double(__double2hiint(x) & 0x7FFFFFFF, __double2loint(x));
   }
   static __device__ __forceinline__ bool neg(double x) { return __double2hiint(x) < 0; }
-  static __device__ __forceinline__ bool live(double ss) {
-    return __double2hiint(ss) > 0x00100000 && __double2hiint(ss) < 0x7FF00000;
-  }
+  static __device__ __forceinline__ bool null(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) <= 0x00100000; }
+  static __device__ __forceinline__ bool finite(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) < 0x7FF00000; }
 };
 
 template <typename C>
@@ -106,7 +97,7 @@ __device__ __forceinline__ C group_sum(C v, unsigned mask) {
 // v_j = x_jj - alpha, alpha = -sign(x_jj) |x_j|, beta = 1 / (|x_j|^2 + |x_jj| |x_j|)) and applies it
 // (v^T a = x_j^T a - alpha a_j, so one pass of dot products serves norm and update). The reflectors go to
 // X, from where the columns of Q, held the same way, take them back in reverse order without a barrier.
-// A null column gives no reflector and R_jj = 0.
+// A null column gives no reflector and R_jj = 0; one whose squared norm is not finite gives NaN.
 //
 // What bounds it is the chain of one step: the barrier (400 cycles), the dot products, two butterflies over
 // LP lanes, root and reciprocal, the update. Finished rows are skipped.
@@ -176,13 +167,14 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
     const C dot = group_sum<C, LP>(d[0] + d[1], 0xffffffffu);
     arow = qshfl(arow, (threadIdx.x & 31 & ~(LP - 1)) + lj);
     const C x0 = xj[jv].e[jh];
-    const bool live = A::live(ss);
+    const bool live = !A::null(ss);
     C alpha = zero, be = zero;
     if (live) {
       const C nrm = A::sqrt(ss);
       alpha = A::neg(x0) ? nrm : -nrm;
       be = A::rcp(A::fma(A::abs(x0), nrm, ss));
     }
+    if (!A::finite(ss)) alpha = be = C(__int_as_float(0x7FC00000));  // NaN, into R and Q: the caller's checks see it
     if (threadIdx.x == 0) diag[j] = alpha, beta[j] = be;
     if (c == j) {  // my rows above j are final, those below stay as the reflector
       mine = live ? x0 - alpha : zero;

@@ -40,3 +40,22 @@ def test_preparation_qr_at_the_edges_of_the_kernels(d, bonds, precision, eps, nu
     got, want = _dense([c.cpu().numpy() for c in C]), _dense(X)
     # each site: at most 60 sweeps of r rotations, or r reflections, of eps each; twice (preparation, compression)
     assert np.linalg.norm(got - want) <= 2 * L * 60 * max(bonds) * eps * np.linalg.norm(want)
+
+
+# the register kernels' FP64 and double-FP32 forms; an entry that is not finite, or whose square overflows, in the
+# column that the first reflector of its site is formed from
+@pytest.mark.parametrize("precision", ["fp64", "tf32x3"])
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 1e200])
+def test_non_finite_core_is_refused(precision, value):
+    rng = np.random.default_rng(3)
+    bonds = (1, 4, 16, 32, 32, 16, 4, 1)
+    A, B = ([rng.standard_normal((bonds[l], 2, 2, bonds[l + 1])) / bonds[l] ** 0.5 for l in range(7)] for _ in range(2))
+    A[3][0, 0, 0, 0] = value
+    A, B = ([torch.from_numpy(x).cuda() for x in X] for X in (A, B))
+    with pytest.raises(ttfit.TTError) as e:
+        f = ttfit.tt_fit_create(A, B, 16, 0.0, "site", precision=precision)
+        try:
+            f.sweep(1)
+        finally:
+            f.destroy()
+    assert e.value.code == ttfit.TT_ERR_NUMERICAL
