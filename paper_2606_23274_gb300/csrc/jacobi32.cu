@@ -55,6 +55,7 @@ __device__ __forceinline__ bool jacobi32_pair(Col32<LP, NV>& x, float& a, float*
   const float g = lanes_sum32<LP>(g0 + g1);
   // the cosine itself: squares of small columns' products would underflow; columns below 1e-16 of the largest stay
   const bool rot = act && a > 1e-32f && b > 1e-32f && fabsf(g) * rsqrtf(a) * rsqrtf(b) > tol;
+  __syncwarp();  // every lane has read the trailers, which lane 0 is about to replace (a shuffle orders no memory)
   if (rot) {
     const float zeta = __fdividef(b - a, 2.f * g);
     const float z2 = fmaf(zeta, zeta, 1.f);  // overflows for columns of very different size: t = 1 / (2 zeta) there

@@ -52,3 +52,13 @@ def test_svd_with_fp32_sweeps_is_as_accurate(r, floor):
     assert np.abs(U[:, :k].T @ U[:, :k] - np.eye(k)).max() <= tol
     assert np.abs(Vt[:k] @ Vt[:k].T - np.eye(k)).max() <= tol
     assert np.abs(S - s[np.argsort(-s)]).max() <= tol
+
+
+@pytest.mark.parametrize("r", [33, 75, 129, 250])
+def test_svd_with_fp32_sweeps_repeats_its_bits(r):
+    """The kernels add in a fixed order and their lanes agree on every rotation: the same input, the same bits."""
+    M = torch.from_numpy(np.random.default_rng(r).standard_normal((r, r))).cuda()
+    first = ttfit.tt_svd_truncated(M, chi_max=r, tau_rel=0.0)
+    for _ in range(8):
+        again = ttfit.tt_svd_truncated(M, chi_max=r, tau_rel=0.0)
+        assert all(torch.equal(a, b) for a, b in zip(first[:3], again[:3]))
