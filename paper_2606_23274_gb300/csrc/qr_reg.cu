@@ -12,7 +12,9 @@ namespace cg = cooperative_groups;
 namespace ttfit {
 
 // Arithmetic of the register QR in its two types. null: the squared norm of a column without a reflector; finite: one
-// that is neither infinite (an entry, or its square) nor NaN.
+// that is neither infinite (an entry, or its square) nor NaN; safe: one that the reflector can be formed from as it is.
+// field: the exponent field of an entry; shift: the power of two by which a column is scaled whose largest field is f
+// and whose squared norm is not safe; scaled: x 2^s.
 template <typename C>
 struct QrArith;
 
@@ -25,6 +27,15 @@ struct QrArith<df32> {
   static __device__ __forceinline__ bool neg(df32 x) { return x.hi < 0.0f; }
   static __device__ __forceinline__ bool null(df32 ss) { return ss.hi <= 0.0f; }
   static __device__ __forceinline__ bool finite(df32 ss) { return isfinite(ss.hi); }
+  static constexpr bool RESCUES = true;
+  // the products' low words are exact to 2^-149: 1024 of them leave 2^-43 of the smallest norm taken as it is at worst
+  static __device__ __forceinline__ bool safe(df32 ss) { return ss.hi >= 0x1p-96f && ss.hi <= 0x1p80f; }
+  static __device__ __forceinline__ int field(df32 x) { return (__float_as_int(x.hi) >> 23) & 0xFF; }
+  static __device__ __forceinline__ int shift(int f) { return f == 0 || f == 0xFF ? 0 : min(max(127 - f, -100), 100); }
+  static __device__ __forceinline__ df32 scaled(df32 x, int s) {
+    const float w = __int_as_float((127 + s) << 23);
+    return df32(x.hi * w, x.lo * w);
+  }
 };
 
 // FP64: the FP64 pipe takes 64 cycles for a warp instruction on this GPU, so square root and reciprocal
@@ -71,6 +82,11 @@ struct QrArith<double> {
   static __device__ __forceinline__ bool neg(double x) { return __double2hiint(x) < 0; }
   static __device__ __forceinline__ bool null(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) <= 0x00100000; }
   static __device__ __forceinline__ bool finite(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) < 0x7FF00000; }
+  static constexpr bool RESCUES = false;
+  static __device__ __forceinline__ bool safe(double) { return true; }
+  static __device__ __forceinline__ int field(double) { return 0; }
+  static __device__ __forceinline__ int shift(int) { return 0; }
+  static __device__ __forceinline__ double scaled(double x, int) { return x; }
 };
 
 template <typename C>
@@ -98,6 +114,10 @@ __device__ __forceinline__ C group_sum(C v, unsigned mask) {
 // (v^T a = x_j^T a - alpha a_j, so one pass of dot products serves norm and update). The reflectors go to
 // X, from where the columns of Q, held the same way, take them back in reverse order without a barrier.
 // A null column gives no reflector and R_jj = 0; one whose squared norm is not finite gives NaN.
+// Where the squared norm is not safe, x_j is first brought near 1 by a power of two, which H does not depend on: in
+// df32 |x_j| < 5e-20 made beta infinite and every later column NaN, and ordinary operators reach that (bond weights
+// 2^-k, from k = 64 on). Every thread sees the same |x_j|^2. The loop stands twice, first without the scaling, up to
+// the first column that needs it: in one loop, at the limit of registers, 512 x 128 df32 took 694 us instead of 628.
 //
 // What bounds it is the chain of one step: the barrier (400 cycles), the dot products, two butterflies over
 // LP lanes, root and reciprocal, the update. Finished rows are skipped.
@@ -121,6 +141,8 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
   const C zero = C(0.0f), one = C(1.0f);
   V a[RP];
   C mine = zero;  // the reflector's entry on the diagonal
+  __shared__ int ups[64];  // per column: the power of two by which its rows from the diagonal on are to be scaled
+  if (l == 0) ups[grp] = 0;
 #pragma unroll
   for (int t = 0; t < RP; ++t)
 #pragma unroll
@@ -141,30 +163,45 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
   cl.sync();  // every CTA runs
   if (c == 0) publish(0);
   cl.sync();
-  for (int j = 0; j < r; ++j) {
-    const V* xj = pub + (j & 1) * LP * RP;
+  // one step; without `rescue` it does nothing and returns false where the column has to be scaled first
+  auto step = [&](auto rescue, int j) -> bool {
+    V* xj = pub + (j & 1) * LP * RP;
     const int jv = j / N, jh = j % N, t0 = jv / LP, lj = jv & (LP - 1);  // row j: element jh of vector t0, lane lj
     V v[RP];
-    C d[2], s[2], arow = zero;
-    d[0] = d[1] = s[0] = s[1] = zero;
+    C ss, dot, arow = zero;
+    int k = 0;  // x_j was scaled by 2^k
+    for (;;) {
+      C d[2], s[2];
+      d[0] = d[1] = s[0] = s[1] = zero;
 #pragma unroll
-    for (int t = 0; t < RP; ++t) {
-      if (t >= t0) {
-        v[t] = xj[l + LP * t];
+      for (int t = 0; t < RP; ++t) {
+        if (t >= t0) {
+          v[t] = xj[l + LP * t];
 #pragma unroll
-        for (int h = 0; h < N; ++h) {
-          d[h & 1] = A::fma(v[t].e[h], a[t].e[h], d[h & 1]);
-          s[h & 1] = A::fma(v[t].e[h], v[t].e[h], s[h & 1]);
+          for (int h = 0; h < N; ++h) {
+            d[h & 1] = A::fma(v[t].e[h], a[t].e[h], d[h & 1]);
+            s[h & 1] = A::fma(v[t].e[h], v[t].e[h], s[h & 1]);
+          }
+        }
+        if (t == t0) {
+#pragma unroll
+          for (int h = 0; h < N; ++h)
+            if (h == jh) arow = a[t].e[h];
         }
       }
-      if (t == t0) {
-#pragma unroll
-        for (int h = 0; h < N; ++h)
-          if (h == jh) arow = a[t].e[h];
-      }
+      ss = group_sum<C, LP>(s[0] + s[1], 0xffffffffu);
+      dot = group_sum<C, LP>(d[0] + d[1], 0xffffffffu);
+      if (A::safe(ss) || k != 0) break;  // the same in every thread
+      if constexpr (!decltype(rescue)::value) return false;
+      C* x = (C*)xj;
+      int f = 0;
+      for (int i = threadIdx.x & 31; i < N * LP * RP; i += 32) f = max(f, A::field(x[i]));
+      k = A::shift(__reduce_max_sync(0xffffffffu, f));
+      if (k == 0) break;
+      __syncthreads();  // this CTA's copy has been read
+      for (int i = threadIdx.x; i < N * LP * RP; i += blockDim.x) x[i] = A::scaled(x[i], k);
+      __syncthreads();
     }
-    const C ss = group_sum<C, LP>(s[0] + s[1], 0xffffffffu);
-    const C dot = group_sum<C, LP>(d[0] + d[1], 0xffffffffu);
     arow = qshfl(arow, (threadIdx.x & 31 & ~(LP - 1)) + lj);
     const C x0 = xj[jv].e[jh];
     const bool live = !A::null(ss);
@@ -178,6 +215,7 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
     if (threadIdx.x == 0) diag[j] = alpha, beta[j] = be;
     if (c == j) {  // my rows above j are final, those below stay as the reflector
       mine = live ? x0 - alpha : zero;
+      if (l == 0) ups[grp] = k;
     } else if (live && c > j && c < p) {
       const C v0 = x0 - alpha;
       const C w = -(be * A::fma(-alpha, arow, dot));
@@ -193,19 +231,28 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
     }
     if (j + 1 < r && c == j + 1) publish(j + 1);
     cl.sync();
+    return true;
+  };
+  int j = 0;
+#pragma unroll 1
+  while (j < r && step(std::false_type{}, j)) ++j;
+  if constexpr (A::RESCUES) {
+#pragma unroll 1
+    for (; j < r; ++j) step(std::true_type{}, j);
   }
   // R (r x p, ld r) with diag >= 0, and the reflectors in place of X (not earlier: a barrier would wait
   // for stores to global memory at every step)
   if (c < p) {
+    const int up = ups[grp];
     const bool dead = c < r && beta[c] == zero;  // a null column
 #pragma unroll
     for (int t = 0; t < RP; ++t)
 #pragma unroll
       for (int h = 0; h < N; ++h) {
         const int i = N * (l + LP * t) + h;
-        if (c < r && i < q) Hg[(size_t)c * q + i] = i > c ? (dead ? zero : a[t].e[h]) : (i == c ? mine : zero);
+        if (c < r && i < q) Hg[(size_t)c * q + i] = i > c ? (dead ? zero : A::scaled(a[t].e[h], up)) : (i == c ? mine : zero);
         if (i >= r) continue;
-        const C x = i > c ? zero : (i == c ? diag[c] : a[t].e[h]);
+        const C x = i > c ? zero : (i == c ? A::scaled(diag[c], -up) : a[t].e[h]);
         Rg[(size_t)c * r + i] = S(A::neg(diag[i]) ? -x : x);
       }
   }

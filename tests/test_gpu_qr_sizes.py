@@ -9,7 +9,9 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
+from mpo_props import diff_norm, norm2  # noqa: E402
 from paper_2606_23274_gb300 import ttfit  # noqa: E402
+from paper_2606_23274_gb300.synth import kron_sum_mpo  # noqa: E402
 
 
 def _dense(cores):
@@ -59,3 +61,31 @@ def test_non_finite_core_is_refused(precision, value):
         finally:
             f.destroy()
     assert e.value.code == ttfit.TT_ERR_NUMERICAL
+
+
+def _norm2_of_a_sweep(A, B, chi, precision):
+    f = ttfit.tt_fit_create(A, B, chi, 0.0, "site", update="rsvd", oversample=10, seed=0, precision=precision, conv_tol=0.0)
+    n2 = f.sweep(1)["norm2_C"]
+    f.destroy()
+    return n2
+
+
+# bond weights 2^-k and 0.7^k: what is left of the last columns of a site lies between 4e-23 and 5e-20, where the
+# square is in the range of FP32 and its reciprocal is not
+@pytest.mark.parametrize("L,K,decay", [(20, 64, 0.5), (30, 128, 0.7)])
+def test_graded_chains_are_prepared(L, K, decay):
+    A, B = ([torch.from_numpy(x).cuda() for x in kron_sum_mpo(L, K, 0, w, decay=decay)] for w in (0, 1))
+    C = ttfit.tt_mpo_compress(A, K, 0.0, precision="df32")
+    assert diff_norm(C, A) <= 2 * L * 60 * K * 2.0 ** -44 * norm2(A) ** 0.5  # as above
+    want = _norm2_of_a_sweep(A, B, K, "fp64")
+    for precision, eps in (("df32", 2.0 ** -44), ("tf32x3", 2.0 ** -21)):
+        assert abs(_norm2_of_a_sweep(A, B, K, precision) - want) <= 2 * (2 * L * 60 * K * eps) * want
+
+
+# a site whose columns all have squares below or above what FP32 holds; below, it came out as a site without rank
+@pytest.mark.parametrize("scale", [2.0 ** -66, 2.0 ** -100, 2.0 ** 66, 2.0 ** 100])
+def test_preparation_does_not_depend_on_the_scale_of_a_site(scale):
+    A, B = ([torch.from_numpy(x).cuda() for x in kron_sum_mpo(12, 32, 0, w)] for w in (0, 1))
+    want = _norm2_of_a_sweep(A, B, 32, "df32")
+    A[0] = A[0] * scale
+    assert abs(_norm2_of_a_sweep(A, B, 32, "df32") - want * scale ** 2) <= 2 * (2 * 12 * 60 * 32 * 2.0 ** -44) * want * scale ** 2
