@@ -14,7 +14,8 @@ namespace ttfit {
 // Arithmetic of the register QR in its two types. null: the squared norm of a column without a reflector; finite: one
 // that is neither infinite (an entry, or its square) nor NaN; safe: one that the reflector can be formed from as it is.
 // field: the exponent field of an entry; shift: the power of two by which a column is scaled whose largest field is f
-// and whose squared norm is not safe; scaled: x 2^s.
+// and whose squared norm is not safe; scaled: x 2^s. lift: the power of two by which a column of X is scaled on
+// loading, f the largest exponent field (FP64) of its entries.
 template <typename C>
 struct QrArith;
 
@@ -27,7 +28,8 @@ struct QrArith<df32> {
   static __device__ __forceinline__ bool neg(df32 x) { return x.hi < 0.0f; }
   static __device__ __forceinline__ bool null(df32 ss) { return ss.hi <= 0.0f; }
   static __device__ __forceinline__ bool finite(df32 ss) { return isfinite(ss.hi); }
-  static constexpr bool RESCUES = true;
+  static constexpr bool RESCUES = true, LIFTS = true;
+  static __device__ __forceinline__ int lift(int f) { return f == 0 || f == 0x7FF ? 0 : 1023 - f; }
   // the products' low words are exact to 2^-149: 1024 of them leave 2^-43 of the smallest norm taken as it is at worst
   static __device__ __forceinline__ bool safe(df32 ss) { return ss.hi >= 0x1p-96f && ss.hi <= 0x1p80f; }
   static __device__ __forceinline__ int field(df32 x) { return (__float_as_int(x.hi) >> 23) & 0xFF; }
@@ -82,12 +84,22 @@ struct QrArith<double> {
   static __device__ __forceinline__ bool neg(double x) { return __double2hiint(x) < 0; }
   static __device__ __forceinline__ bool null(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) <= 0x00100000; }
   static __device__ __forceinline__ bool finite(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) < 0x7FF00000; }
-  static constexpr bool RESCUES = false;
+  static constexpr bool RESCUES = false, LIFTS = false;
+  static __device__ __forceinline__ int lift(int) { return 0; }
   static __device__ __forceinline__ bool safe(double) { return true; }
   static __device__ __forceinline__ int field(double) { return 0; }
   static __device__ __forceinline__ int shift(int) { return 0; }
   static __device__ __forceinline__ double scaled(double x, int) { return x; }
 };
+
+// x 2^s by the bits; zero below the normal numbers
+__device__ __forceinline__ double shift_bits(double x, int s) {
+  const int hi = __double2hiint(x), f = (hi >> 20) & 0x7FF, g = f + s;
+  if (f == 0x7FF || s == 0) return x;
+  if (f == 0 || g <= 0) return 0.0;
+  if (g >= 0x7FF) return __hiloint2double((hi & (int)0x80000000) | 0x7FF00000, 0);
+  return __hiloint2double(hi + (int)((unsigned)s << 20), __double2loint(x));
+}
 
 template <typename C>
 struct __align__(16) Vec16 {
@@ -118,6 +130,8 @@ __device__ __forceinline__ C group_sum(C v, unsigned mask) {
 // df32 |x_j| < 5e-20 made beta infinite and every later column NaN, and ordinary operators reach that (bond weights
 // 2^-k, from k = 64 on). Every thread sees the same |x_j|^2. The loop stands twice, first without the scaling, up to
 // the first column that needs it: in one loop, at the limit of registers, 512 x 128 df32 took 694 us instead of 628.
+// The columns of X are each brought near 1 on loading, and those of R back, so that df32, whose exponents are FP32's,
+// takes the range of FP64 (a site below 1e-45 came out null, one above 3e38 was refused).
 //
 // What bounds it is the chain of one step: the barrier (400 cycles), the dot products, two butterflies over
 // LP lanes, root and reciprocal, the update. Finished rows are skipped.
@@ -141,15 +155,25 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
   const C zero = C(0.0f), one = C(1.0f);
   V a[RP];
   C mine = zero;  // the reflector's entry on the diagonal
-  __shared__ int ups[64];  // per column: the power of two by which its rows from the diagonal on are to be scaled
+  // per column: the powers of two by which it was scaled on loading, and its rows from the diagonal on are to be
+  __shared__ int lifts[64], ups[64];
   if (l == 0) ups[grp] = 0;
+  {
+    int f = 0;
+    if (A::LIFTS && c < p)
+      for (int i = l; i < q; i += LP) f = max(f, (__double2hiint(Xg[(size_t)c * q + i]) >> 20) & 0x7FF);
 #pragma unroll
-  for (int t = 0; t < RP; ++t)
+    for (int o = LP / 2; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
+    const int lift = A::lift(f);
+    if (l == 0) lifts[grp] = lift;
 #pragma unroll
-    for (int h = 0; h < N; ++h) {
-      const int i = N * (l + LP * t) + h;
-      a[t].e[h] = (c < p && i < q) ? C(Xg[(size_t)c * q + i]) : zero;
-    }
+    for (int t = 0; t < RP; ++t)
+#pragma unroll
+      for (int h = 0; h < N; ++h) {
+        const int i = N * (l + LP * t) + h;
+        a[t].e[h] = (c < p && i < q) ? C(shift_bits(Xg[(size_t)c * q + i], lift)) : zero;
+      }
+  }
   auto publish = [&](int j) {  // my column (j) to every CTA, zeros above row j
     V* dst = pub + (j & 1) * LP * RP + l;
 #pragma unroll
@@ -243,7 +267,7 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
   // R (r x p, ld r) with diag >= 0, and the reflectors in place of X (not earlier: a barrier would wait
   // for stores to global memory at every step)
   if (c < p) {
-    const int up = ups[grp];
+    const int up = ups[grp], lift = lifts[grp];
     const bool dead = c < r && beta[c] == zero;  // a null column
 #pragma unroll
     for (int t = 0; t < RP; ++t)
@@ -253,7 +277,7 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
         if (c < r && i < q) Hg[(size_t)c * q + i] = i > c ? (dead ? zero : A::scaled(a[t].e[h], up)) : (i == c ? mine : zero);
         if (i >= r) continue;
         const C x = i > c ? zero : (i == c ? A::scaled(diag[c], -up) : a[t].e[h]);
-        Rg[(size_t)c * r + i] = S(A::neg(diag[i]) ? -x : x);
+        Rg[(size_t)c * r + i] = shift_bits(S(A::neg(diag[i]) ? -x : x), -lift);
       }
   }
   if (Qg != nullptr) {  // uniform

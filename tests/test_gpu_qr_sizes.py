@@ -82,8 +82,9 @@ def test_graded_chains_are_prepared(L, K, decay):
         assert abs(_norm2_of_a_sweep(A, B, K, precision) - want) <= 2 * (2 * L * 60 * K * eps) * want
 
 
-# a site whose columns all have squares below or above what FP32 holds; below, it came out as a site without rank
-@pytest.mark.parametrize("scale", [2.0 ** -66, 2.0 ** -100, 2.0 ** 66, 2.0 ** 100])
+# a site whose columns all have squares below or above what FP32 holds, or lie themselves outside of it; below, it came
+# out as a site without rank
+@pytest.mark.parametrize("scale", [2.0 ** -66, 2.0 ** -100, 2.0 ** 66, 2.0 ** 100, 2.0 ** -200, 2.0 ** -450, 2.0 ** 300])
 def test_preparation_does_not_depend_on_the_scale_of_a_site(scale):
     A, B = ([torch.from_numpy(x).cuda() for x in kron_sum_mpo(12, 32, 0, w)] for w in (0, 1))
     want = _norm2_of_a_sweep(A, B, 32, "df32")
