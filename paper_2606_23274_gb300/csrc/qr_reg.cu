@@ -28,7 +28,7 @@ struct QrArith<df32> {
   static __device__ __forceinline__ bool neg(df32 x) { return x.hi < 0.0f; }
   static __device__ __forceinline__ bool null(df32 ss) { return ss.hi <= 0.0f; }
   static __device__ __forceinline__ bool finite(df32 ss) { return isfinite(ss.hi); }
-  static constexpr bool RESCUES = true, LIFTS = true;
+  static constexpr bool RESCUES = true;
   static __device__ __forceinline__ int lift(int f) { return f == 0 || f == 0x7FF ? 0 : 1023 - f; }
   // the products' low words are exact to 2^-149: 1024 of them leave 2^-43 of the smallest norm taken as it is at worst
   static __device__ __forceinline__ bool safe(df32 ss) { return ss.hi >= 0x1p-96f && ss.hi <= 0x1p80f; }
@@ -84,8 +84,9 @@ struct QrArith<double> {
   static __device__ __forceinline__ bool neg(double x) { return __double2hiint(x) < 0; }
   static __device__ __forceinline__ bool null(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) <= 0x00100000; }
   static __device__ __forceinline__ bool finite(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) < 0x7FF00000; }
-  static constexpr bool RESCUES = false, LIFTS = false;
-  static __device__ __forceinline__ int lift(int) { return 0; }
+  // only columns below 2^-300, whose squares lose accuracy; an entry whose square overflows is refused
+  static constexpr bool RESCUES = false;
+  static __device__ __forceinline__ int lift(int f) { return f == 0 || f > 723 ? 0 : 1023 - f; }
   static __device__ __forceinline__ bool safe(double) { return true; }
   static __device__ __forceinline__ int field(double) { return 0; }
   static __device__ __forceinline__ int shift(int) { return 0; }
@@ -131,7 +132,8 @@ __device__ __forceinline__ C group_sum(C v, unsigned mask) {
 // 2^-k, from k = 64 on). Every thread sees the same |x_j|^2. The loop stands twice, first without the scaling, up to
 // the first column that needs it: in one loop, at the limit of registers, 512 x 128 df32 took 694 us instead of 628.
 // The columns of X are each brought near 1 on loading, and those of R back, so that df32, whose exponents are FP32's,
-// takes the range of FP64 (a site below 1e-45 came out null, one above 3e38 was refused).
+// takes the range of FP64 (a site below 1e-45 came out null, one above 3e38 was refused); in FP64 the very small ones
+// (below 1.5e-154, where the square is not a normal number, they came out null).
 //
 // What bounds it is the chain of one step: the barrier (400 cycles), the dot products, two butterflies over
 // LP lanes, root and reciprocal, the update. Finished rows are skipped.
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
   if (l == 0) ups[grp] = 0;
   {
     int f = 0;
-    if (A::LIFTS && c < p)
+    if (c < p)
       for (int i = l; i < q; i += LP) f = max(f, (__double2hiint(Xg[(size_t)c * q + i]) >> 20) & 0x7FF);
 #pragma unroll
     for (int o = LP / 2; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));

@@ -90,3 +90,19 @@ def test_preparation_does_not_depend_on_the_scale_of_a_site(scale):
     want = _norm2_of_a_sweep(A, B, 32, "df32")
     A[0] = A[0] * scale
     assert abs(_norm2_of_a_sweep(A, B, 32, "df32") - want * scale ** 2) <= 2 * (2 * 12 * 60 * 32 * 2.0 ** -44) * want * scale ** 2
+
+
+# columns whose squares are not normal FP64 numbers, or zero
+@pytest.mark.parametrize("e", [525, 600, 900])
+def test_preparation_takes_sites_whose_squares_underflow(e):
+    A, B = ([torch.from_numpy(x).cuda() for x in kron_sum_mpo(12, 32, 0, w)] for w in (0, 1))
+    A[0] = A[0] * 2.0 ** -e
+    f = ttfit.tt_fit_create(A, B, 32, 0.0, "site", update="rsvd", oversample=10, seed=0, precision="fp64", conv_tol=0.0)
+    f.sweep(1)
+    C = f.result(torch.float64)
+    f.destroy()
+    centre = min(range(12), key=lambda l: float(C[l].abs().max()))
+    C[centre] = C[centre] * 2.0 ** e
+    A[0] = A[0] * 2.0 ** e
+    want = _norm2_of_a_sweep(A, B, 32, "fp64")
+    assert abs(norm2(C) - want) <= 2 * (2 * 12 * 60 * 32 * 2.0 ** -52) * want
