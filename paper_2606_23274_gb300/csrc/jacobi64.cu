@@ -5,6 +5,7 @@
 #include <cfloat>
 #include "common.cuh"
 #include "kernels.h"
+#include "scalar_ops.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -28,6 +29,9 @@ namespace ttfit {
 //    (1973)): with x = dx x~, y = dy y~ a rotation is x~ -= (t dy / dx) y~,
 //    y~ += (t dx / dy) x~, two multiply-adds a row instead of four operations; the
 //    scales take the factor cos and are multiplied in once a sweep.
+//  * A very large or small W is brought to exponent 0 by a power of two while it lies in shared memory, and S
+//    back: squared norms and products of two of them must neither overflow nor vanish (from entries of 1e77 and
+//    1e-77 on no pair rotated any more, and the norms of the columns were returned as singular values).
 // ---------------------------------------------------------------------------
 struct Rot64 {
   double t, cs, s;  // tangent, cosine, 1 + t^2
@@ -157,7 +161,7 @@ __global__ void __launch_bounds__(1024)
   double* buf = (double*)j64s;                                // [nbuf][2 slots][b][ld]
   int* ids = (int*)(buf + (size_t)nbuf * 2 * b * ld);         // [nbuf][2 slots][b] global column or -1
   double* nrm = (double*)(ids + 4 * b + 4);                   // [2 slots][b] final column norms
-  __shared__ int flag[2];
+  __shared__ int flag[2], top;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   constexpr int G = 32 / LP;
   const int grp = warp * G + lane / LP, ng = nw * G, l = lane & (LP - 1);
@@ -165,6 +169,9 @@ __global__ void __launch_bounds__(1024)
   auto cid = [&](int bi, int sl, int k) -> int& { return ids[(bi * 2 + sl) * b + k]; };
   const double tol2 = tol * tol;
 
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
+  int field = 0;  // largest exponent field of my entries of W
   for (int sl = 0; sl < 2; ++sl) {  // CTA c holds the blocks at positions c and P-1-c
     const int blk = sl == 0 ? rank : P - 1 - rank;
     for (int k = 0; k < b; ++k) {
@@ -174,15 +181,30 @@ __global__ void __launch_bounds__(1024)
       for (int r = threadIdx.x; r < ld; r += blockDim.x) {
         double v = 0.0;
         if (r == ld - 3 || r == ld - 2) v = 1.0;
-        else if (gid < p && r < q) v = Win[(size_t)gid * q + r];
-        else if (gid < p && r >= qs && r - qs < p && r < ld - J64_TAIL)
+        else if (gid < p && r < q) {
+          v = Win[(size_t)gid * q + r];
+          field = max(field, (__double2hiint(v) >> 20) & 0x7FF);
+        } else if (gid < p && r >= qs && r - qs < p && r < ld - J64_TAIL)
           v = Vin ? Vin[(size_t)gid * p + r - qs] : (r - qs == gid ? 1.0 : 0.0);
         x[r] = v;
       }
     }
   }
   if (threadIdx.x < 2) flag[threadIdx.x] = 0;
+  field = __reduce_max_sync(0xffffffffu, field);
+  if (lane == 0) atomicMax(&top, field);
   cl.sync();
+  field = __reduce_max_sync(0xffffffffu, lane < NC ? *cl.map_shared_rank(&top, lane) : 0);
+  // not where an entry is not finite, and not within 2^-64 .. 2^64, where it changes nothing
+  const int shift = field == 0 || field == 0x7FF || abs(field - 1023) <= 64 ? 0 : 1023 - field;
+  if (shift != 0) {
+    for (int sl = 0; sl < 2; ++sl)
+      for (int k = 0; k < b; ++k) {
+        double* x = col(0, sl, k);
+        for (int r = threadIdx.x; r < q; r += blockDim.x) x[r] = shift_bits(x[r], shift);
+      }
+    __syncthreads();
+  }
 
   int cur = 0, sweep = 0;
   // multiply the scales into the columns and recompute |w|^2
@@ -292,7 +314,7 @@ __global__ void __launch_bounds__(1024)
     for (int r = lane; r < q; r += 32) Uo[(size_t)rk * q + r] = x[r] * inv;
     if (want_v)
       for (int r = lane; r < p; r += 32) Vo[(size_t)rk * p + r] = x[qs + r];
-    if (lane == 0) So[rk] = v;
+    if (lane == 0) So[rk] = scalbn(v, -shift);
   }
   cl.sync();  // no CTA leaves while another may still read its shared memory
 }
@@ -448,7 +470,8 @@ cudaError_t svd_tall64(int q, int p, double* X, double* T1, double* T2, double* 
   cudaError_t e = cudaSuccess;
   if (p >= 32 && q <= 1024 && (e = jacobi64_plan(p, p, true, st, plan)) != cudaSuccess) return e;
   if (!plan.kern) return jacobi_svd<double, double>(q, p, X, T1, Sv, V, T2, max_sweeps, errw, st);
-  e = qr_householder<double, double>(q, p, X, T1, T2, st);  // Q: T1, R: T2
+  e = qr_reg64(q, p, X, T1, T2, st, true);  // Q: T1, R: T2
+  if (e == cudaErrorNotSupported) e = qr_householder<double, double>(q, p, X, T1, T2, st);
   if (e != cudaSuccess) return e;
   const IdxMap one = IdxMap::lin(1), row = IdxMap::lin(p);
   if ((e = copy_map<double, double>(p, p, T2, one, row, X, row, one, 1.0, st)) != cudaSuccess) return e;

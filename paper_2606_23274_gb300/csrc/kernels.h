@@ -74,8 +74,9 @@ cudaError_t qr_householder(int q, int p, S* X, S* Q, S* R, cudaStream_t st);
 cudaError_t qr_householder_df32(int q, int p, double* X, double* Q, double* R, cudaStream_t st);
 
 // The same with the columns in registers (qr_reg.cu), which the two above take where it fits (Q may be
-// null); cudaErrorNotSupported otherwise.
-cudaError_t qr_reg64(int q, int p, double* X, double* Q, double* R, cudaStream_t st);
+// null); cudaErrorNotSupported otherwise. any_scale: large columns are scaled too, where otherwise one whose
+// squared norm overflows gives NaN.
+cudaError_t qr_reg64(int q, int p, double* X, double* Q, double* R, cudaStream_t st, bool any_scale = false);
 cudaError_t qr_reg_df32(int q, int p, double* X, double* Q, double* R, cudaStream_t st);
 
 // One-sided Jacobi SVD of the q x p column-major W (q >= p, ld q; overwritten):

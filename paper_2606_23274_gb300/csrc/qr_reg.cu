@@ -29,7 +29,7 @@ struct QrArith<df32> {
   static __device__ __forceinline__ bool null(df32 ss) { return ss.hi <= 0.0f; }
   static __device__ __forceinline__ bool finite(df32 ss) { return isfinite(ss.hi); }
   static constexpr bool RESCUES = true;
-  static __device__ __forceinline__ int lift(int f) { return f == 0 || f == 0x7FF ? 0 : 1023 - f; }
+  static __device__ __forceinline__ int lift(int f, int) { return f == 0 || f == 0x7FF ? 0 : 1023 - f; }
   // the products' low words are exact to 2^-149: 1024 of them leave 2^-43 of the smallest norm taken as it is at worst
   static __device__ __forceinline__ bool safe(df32 ss) { return ss.hi >= 0x1p-96f && ss.hi <= 0x1p80f; }
   static __device__ __forceinline__ int field(df32 x) { return (__float_as_int(x.hi) >> 23) & 0xFF; }
@@ -84,23 +84,16 @@ struct QrArith<double> {
   static __device__ __forceinline__ bool neg(double x) { return __double2hiint(x) < 0; }
   static __device__ __forceinline__ bool null(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) <= 0x00100000; }
   static __device__ __forceinline__ bool finite(double ss) { return (__double2hiint(ss) & 0x7FFFFFFF) < 0x7FF00000; }
-  // only columns below 2^-300, whose squares lose accuracy; an entry whose square overflows is refused
+  // only columns below 2^-300, whose squares lose accuracy, and those above the field `top`
   static constexpr bool RESCUES = false;
-  static __device__ __forceinline__ int lift(int f) { return f == 0 || f > 723 ? 0 : 1023 - f; }
+  static __device__ __forceinline__ int lift(int f, int top) {
+    return f == 0 || f == 0x7FF || (f > 723 && f <= top) ? 0 : 1023 - f;
+  }
   static __device__ __forceinline__ bool safe(double) { return true; }
   static __device__ __forceinline__ int field(double) { return 0; }
   static __device__ __forceinline__ int shift(int) { return 0; }
   static __device__ __forceinline__ double scaled(double x, int) { return x; }
 };
-
-// x 2^s by the bits; zero below the normal numbers
-__device__ __forceinline__ double shift_bits(double x, int s) {
-  const int hi = __double2hiint(x), f = (hi >> 20) & 0x7FF, g = f + s;
-  if (f == 0x7FF || s == 0) return x;
-  if (f == 0 || g <= 0) return 0.0;
-  if (g >= 0x7FF) return __hiloint2double((hi & (int)0x80000000) | 0x7FF00000, 0);
-  return __hiloint2double(hi + (int)((unsigned)s << 20), __double2loint(x));
-}
 
 template <typename C>
 struct __align__(16) Vec16 {
@@ -133,13 +126,13 @@ __device__ __forceinline__ C group_sum(C v, unsigned mask) {
 // the first column that needs it: in one loop, at the limit of registers, 512 x 128 df32 took 694 us instead of 628.
 // The columns of X are each brought near 1 on loading, and those of R back, so that df32, whose exponents are FP32's,
 // takes the range of FP64 (a site below 1e-45 came out null, one above 3e38 was refused); in FP64 the very small ones
-// (below 1.5e-154, where the square is not a normal number, they came out null).
+// (below 1.5e-154, where the square is not a normal number, they came out null) and, for decompositions, very large.
 //
 // What bounds it is the chain of one step: the barrier (400 cycles), the dot products, two butterflies over
 // LP lanes, root and reciprocal, the update. Finished rows are skipped.
 template <typename S, typename C, int LP, int RP>
 __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
-    qr_reg_kernel(int q, int p, S* __restrict__ Xg, S* __restrict__ Qg, S* __restrict__ Rg) {
+    qr_reg_kernel(int q, int p, int top, S* __restrict__ Xg, S* __restrict__ Qg, S* __restrict__ Rg) {
   using A = QrArith<C>;
   using V = Vec16<C>;
   constexpr int N = V::N;
@@ -166,7 +159,7 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
       for (int i = l; i < q; i += LP) f = max(f, (__double2hiint(Xg[(size_t)c * q + i]) >> 20) & 0x7FF);
 #pragma unroll
     for (int o = LP / 2; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
-    const int lift = A::lift(f);
+    const int lift = A::lift(f, top);
     if (l == 0) lifts[grp] = lift;
 #pragma unroll
     for (int t = 0; t < RP; ++t)
@@ -345,7 +338,7 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
 }
 
 template <typename S, typename C>
-cudaError_t qr_reg_launch(int nc, int lp, int q, int p, S* X, S* Q, S* R, cudaStream_t st) {
+cudaError_t qr_reg_launch(int nc, int lp, int q, int p, int top, S* X, S* Q, S* R, cudaStream_t st) {
   constexpr int N = Vec16<C>::N;
   const int threads = ((p + nc - 1) / nc * lp + 31) / 32 * 32;
   const int rp = q <= 4 * N * lp ? 4 : q <= 8 * N * lp ? 8 : 16;
@@ -377,7 +370,7 @@ cudaError_t qr_reg_launch(int nc, int lp, int q, int p, S* X, S* Q, S* R, cudaSt
       }
     }
     ++tl_launches;
-    e = cudaLaunchKernelEx(&cfg, kern, q, p, X, Q, R);
+    e = cudaLaunchKernelEx(&cfg, kern, q, p, top, X, Q, R);
     return e != cudaSuccess ? e : cudaGetLastError();
   };
   if (lp == 8)
@@ -391,20 +384,21 @@ cudaError_t qr_reg_launch(int nc, int lp, int q, int p, S* X, S* Q, S* R, cudaSt
 // rows marked *, the one-CTA kernel takes): 64 x 20 *298: 4 CTAs of 8 lanes 72; 64 x 64 *1203: 8 x 8 209;
 // 100 x 37 *620: 8 x 16 138; 128 x 128 1397: 8 x 16 630; 256 x 74 934: 8 x 16 444, 16 x 32 328;
 // 512 x 128 2312: 8 x 16 1825, 16 x 32 1088.
-cudaError_t qr_reg64(int q, int p, double* X, double* Q, double* R, cudaStream_t st) {
+cudaError_t qr_reg64(int q, int p, double* X, double* Q, double* R, cudaStream_t st, bool any_scale) {
+  const int top = any_scale ? 1023 + 300 : 0x7FE;
   const int lp = q <= 64 ? 8 : q <= 128 ? 16 : 32;
   if (q > 128 && p > 32) {
-    const cudaError_t e = qr_reg_launch<double, double>(16, lp, q, p, X, Q, R, st);
+    const cudaError_t e = qr_reg_launch<double, double>(16, lp, q, p, top, X, Q, R, st);
     if (e != cudaErrorNotSupported) return e;
   }
-  return qr_reg_launch<double, double>(p <= 32 ? 4 : 8, lp, q, p, X, Q, R, st);
+  return qr_reg_launch<double, double>(p <= 32 ? 4 : 8, lp, q, p, top, X, Q, R, st);
 }
 
 // Double-FP32 arithmetic on FP64 storage. 128 x 128: 888 us by the blocked kernel, 284 here (8 CTAs of
 // 16 lanes); 256 x 64: 420, 169 (8 x 32); 512 x 128: 1199, 666 (8 x 32). Clusters of 16 take 578 for the
 // last, but two chains and the random guess prepare at once, and 8 leave them room.
 cudaError_t qr_reg_df32(int q, int p, double* X, double* Q, double* R, cudaStream_t st) {
-  return qr_reg_launch<double, df32>(8, q <= 128 ? 16 : 32, q, p, X, Q, R, st);
+  return qr_reg_launch<double, df32>(8, q <= 128 ? 16 : 32, q, p, 0, X, Q, R, st);
 }
 
 }  // namespace ttfit

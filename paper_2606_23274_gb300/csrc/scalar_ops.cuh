@@ -63,4 +63,13 @@ __device__ __forceinline__ float rot_rsqrt(float x) {
   return fmaf(0.5f * r, fmaf(-x * r, r, 1.f), r);
 }
 
+// x 2^s by the bits; zero below the normal numbers
+__device__ __forceinline__ double shift_bits(double x, int s) {
+  const int hi = __double2hiint(x), f = (hi >> 20) & 0x7FF, g = f + s;
+  if (f == 0x7FF || s == 0) return x;
+  if (f == 0 || g <= 0) return 0.0;
+  if (g >= 0x7FF) return __hiloint2double((hi & (int)0x80000000) | 0x7FF00000, 0);
+  return __hiloint2double(hi + (int)((unsigned)s << 20), __double2loint(x));
+}
+
 }  // namespace ttfit

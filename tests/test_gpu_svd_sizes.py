@@ -62,3 +62,18 @@ def test_svd_with_fp32_sweeps_repeats_its_bits(r):
     for _ in range(8):
         again = ttfit.tt_svd_truncated(M, chi_max=r, tau_rel=0.0)
         assert all(torch.equal(a, b) for a, b in zip(first[:3], again[:3]))
+
+
+# one CTA, 8 and 16 CTAs, the long side on either hand; entries whose squares, or their products, leave the range
+@pytest.mark.parametrize("m,n", [(24, 16), (64, 40), (40, 64), (130, 120)])
+@pytest.mark.parametrize("scale", [1e80, 1e-80, 1e140, 1e-140])
+def test_svd_does_not_depend_on_the_scale(m, n, scale):
+    rng = np.random.default_rng(m * 2000 + n)
+    r = min(m, n)
+    M = rng.standard_normal((m, n))
+    U, S, Vt, _ = ttfit.tt_svd_truncated(M * scale, chi_max=r, tau_rel=0.0)
+    U, S, Vt = U.cpu().numpy(), S.cpu().numpy() / scale, Vt.cpu().numpy()
+    tol = 60 * r * EPS  # as above
+    assert np.linalg.norm(U * S[None, :] @ Vt - M) <= tol * np.linalg.norm(M)
+    assert np.abs(U.T @ U - np.eye(r)).max() <= tol and np.abs(Vt @ Vt.T - np.eye(r)).max() <= tol
+    assert np.abs(S - np.linalg.svd(M, compute_uv=False)).max() <= tol * np.linalg.norm(M)

@@ -208,3 +208,17 @@ def test_zipup_guess_with_projection_follows_oracle(gauge):
             assert abs(rep["norm2_C"] - want) <= 1e-9 * want, (s, rep["norm2_C"], want)
     finally:
         f.destroy()
+
+
+# M_l of 64 and 400 rows (Jacobi), and of 1600 (its Gram matrix, whose entries are squares already)
+@pytest.mark.parametrize("K,chi", [(8, 20), (20, 40), (40, 40)])
+@pytest.mark.parametrize("e", [-260, -135, 130, 260])
+def test_zipup_does_not_depend_on_the_scale(K, chi, e):
+    """Every step of the zip-up is linear or scale-free: a power of two in the last core of A comes out in the first
+    of C, and all other bits are the same."""
+    A, B = (kron_sum_mpo(6, K, 0, w) for w in (0, 1))
+    kw = dict(update="rsvd", oversample=10, seed=5, precision="fp64", prepare_inputs=0)
+    R = ttfit.tt_mpo_zipup(A, B, chi, 0.0, **kw)
+    A[-1] = A[-1] * 2.0 ** e
+    C = ttfit.tt_mpo_zipup(A, B, chi, 0.0, **kw)
+    assert torch.equal(C[0] * 2.0 ** -e, R[0]) and all(torch.equal(c, r) for c, r in zip(C[1:], R[1:]))
