@@ -357,7 +357,8 @@ tt_status tt_mpo_grad(const tt_mpo_desc* A, const tt_mpo_desc* B, const tt_mpo_d
  * scratch from the block cache (tt_device_cache_release), runs on `stream`
  * (cudaStream_t, NULL = default) and synchronises it. Errors: TT_ERR_INVALID_ARGUMENT (NULL pointer,
  * non-positive size, r > 1024), TT_ERR_OUT_OF_MEMORY, TT_ERR_CUDA,
- * TT_ERR_NUMERICAL (non-finite input, no convergence). */
+ * TT_ERR_NUMERICAL (non-finite input, a singular value beyond FP64's range,
+ * no convergence). */
 tt_status tt_svd_truncated(const double* M, int m, int n, int chi_max, double tau_rel, double* U, double* S,
                            double* Vt, int* k_out, void* stream);
 

@@ -115,7 +115,7 @@ cudaError_t frob_norm(const T* x, long long n, double* out, uint32_t* errw, cuda
 
 // Truncation rule (Sec. 2.3.4): from sorted S (p values), ||M||_F, writes
 // info[0] = k, and dinfo[0] = sum_{j<k} s_j^2, dinfo[1] = sqrt(sum_{j>=k} s_j^2)/||M||_F.
-// With e (device): S and ||M|| are those of 2^-e M and are scaled back first, in place.
+// With e (device): S and ||M|| are those of 2^-e M and are scaled back in place.
 template <typename F>
 cudaError_t truncate_rule(F* S, int p, double* normM, const int* e, double tau_over_L, int chi_max,
                           double cutoff, int* info, double* dinfo, cudaStream_t st);

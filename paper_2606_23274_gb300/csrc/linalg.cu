@@ -1332,14 +1332,7 @@ __global__ void truncate_kernel(F* S, int p, double* normM, const int* e, double
                                 double cutoff, int* info, double* dinfo) {
   const int lane = threadIdx.x;
   const int run = (p + 31) / 32, j0 = min(p, lane * run), j1 = min(p, j0 + run);
-  double nM = *normM;
-  if (e) {  // the decomposition was that of 2^-e M: s_j <- s_j 2^e, ||M|| <- ||M|| 2^e
-    const int ex = *e;
-    for (int j = j0; j < j1; ++j) S[j] = (F)scalbn((double)S[j], ex);
-    nM = scalbn(nM, ex);
-    __syncwarp();
-    if (lane == 0) *normM = nM;
-  }
+  const double nM = *normM;
   double sq = 0.0;  // of my run
   for (int j = j1 - 1; j >= j0; --j) sq += (double)S[j] * (double)S[j];
   int k = min(chi_max, p);
@@ -1372,9 +1365,17 @@ __global__ void truncate_kernel(F* S, int p, double* normM, const int* e, double
   }
   kept = warp_sum(kept);
   disc = warp_sum(disc);
+  // With e the decomposition was that of 2^-e M. The rule above is free of scale and its squares may not be, so that
+  // s_j, ||M|| and the kept weight are scaled back last (e of a null M: any value)
+  const int ex = e ? max(*e, -4096) : 0;
+  if (e) {
+    __syncwarp();  // every lane has read S and ||M||
+    for (int j = j0; j < j1; ++j) S[j] = (F)scalbn((double)S[j], ex);
+    if (lane == 0) *normM = scalbn(nM, ex);
+  }
   if (lane == 0) {
     info[0] = k;
-    dinfo[0] = kept;
+    dinfo[0] = scalbn(kept, 2 * ex);
     dinfo[1] = nM > 0.0 ? sqrt(disc) / nM : 0.0;
   }
 }
@@ -1827,7 +1828,12 @@ __device__ __forceinline__ float scale_pow2<float, double>(double x, int s) { re
 template <>
 __device__ __forceinline__ float scale_pow2<float, df32>(df32 x, int s) { return scalbnf(x.hi, s) + scalbnf(x.lo, s); }
 template <>
-__device__ __forceinline__ double scale_pow2<double, double>(double x, int s) { return scalbn(x, s); }
+__device__ __forceinline__ double scale_pow2<double, double>(double x, int s) {  // normal numbers by their bits
+  const int hi = __double2hiint(x), f = (hi >> 20) & 0x7FF;
+  if ((unsigned)(f - 1) < 2046u && (unsigned)(f + s - 1) < 2046u)
+    return __hiloint2double(hi + (int)((unsigned)s << 20), __double2loint(x));
+  return scalbn(x, s);
+}
 template <>
 __device__ __forceinline__ double scale_pow2<double, df32>(df32 x, int s) { return scalbn((double)x, s); }
 

@@ -28,7 +28,7 @@ size_t svd_info_offset(int m, int n) {
 
 __global__ void svd_outputs_kernel(int m, int n, int tr, const double* __restrict__ Ux, const double* __restrict__ Vx,
                                    const double* __restrict__ Sv, double* __restrict__ U, double* __restrict__ S,
-                                   double* __restrict__ Vt) {
+                                   double* __restrict__ Vt, uint32_t* errw) {
   // X = Ux diag(S) Vx^T with X = M (tr = 0, Ux m x r) or X = M^T (tr = 1, Ux n x r)
   const int r = min(m, n);
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -41,7 +41,10 @@ __global__ void svd_outputs_kernel(int m, int n, int tr, const double* __restric
     const int j = (int)(e / n), c = (int)(e % n);
     Vt[e] = tr ? Ux[(size_t)j * n + c] : Vx[(size_t)j * r + c];
   }
-  for (long long e = t0; e < r; e += stride) S[e] = Sv[e];
+  for (long long e = t0; e < r; e += stride) {
+    S[e] = Sv[e];
+    if (!isfinite(Sv[e])) atomicOr(errw, ERRW_NAN);
+  }
 }
 
 cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, double* U, double* S, double* Vt,
@@ -56,13 +59,16 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   double* nrm = Sv + r;
   double* dinfo = nrm + 1;
   uint32_t* info = (uint32_t*)(dinfo + 2);
+  int* ex = (int*)info + 2;
   cudaError_t e = cudaMemsetAsync(info, 0, 4 * sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
-  // tall orientation, column-major: M^T column-major is M row-major (tr); else transpose
-  if (tr) e = cudaMemcpyAsync(X, M, sizeof(double) * (size_t)m * n, cudaMemcpyDeviceToDevice, st);
-  else e = copy_map<double, double>(m, n, M, IdxMap::lin(n), IdxMap::lin(1), X, IdxMap::lin(1), IdxMap::lin(m), 1.0, st);
-  if (e != cudaSuccess) return e;
-  if ((e = frob_norm<double>(M, (long long)m * n, nrm, info, st)) != cudaSuccess) return e;
+  // X = 2^-ex M, largest entry near 1: its squares stay in range. Tall orientation, column-major: M^T column-major is M
+  // row-major (tr); else transpose
+  double* M1 = tr ? X : Ux;
+  if ((e = scale_norm<double, double>(M, (long long)m * n, M1, ex, nrm, info, st)) != cudaSuccess) return e;
+  if (!tr && (e = copy_map<double, double>(m, n, M1, IdxMap::lin(n), IdxMap::lin(1), X, IdxMap::lin(1), IdxMap::lin(m), 1.0,
+                                           st)) != cudaSuccess)
+    return e;
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -70,11 +76,11 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   if ((e = fix_signs<double>(tr ? r : q, tr ? q : r, r, tr ? Vx : Ux, tr ? r : q, tr ? Ux : Vx, tr ? q : r, st)) !=
       cudaSuccess)
     return e;
-  if ((e = truncate_rule<double>(Sv, r, nrm, nullptr, tau_rel, chi_max, 1e-13, k_dev, dinfo, st)) != cudaSuccess) return e;
+  if ((e = truncate_rule<double>(Sv, r, nrm, ex, tau_rel, chi_max, 1e-13, k_dev, dinfo, st)) != cudaSuccess) return e;
   const long long tot = (long long)q * r;
   const int blocks = (int)std::max<long long>(1, std::min<long long>((tot + 255) / 256, 1024));
   ++tl_launches;
-  svd_outputs_kernel<<<blocks, 256, 0, st>>>(m, n, tr ? 1 : 0, Ux, Vx, Sv, U, S, Vt);
+  svd_outputs_kernel<<<blocks, 256, 0, st>>>(m, n, tr ? 1 : 0, Ux, Vx, Sv, U, S, Vt, info);
   return cudaGetLastError();
 }
 

@@ -77,3 +77,34 @@ def test_svd_does_not_depend_on_the_scale(m, n, scale):
     assert np.linalg.norm(U * S[None, :] @ Vt - M) <= tol * np.linalg.norm(M)
     assert np.abs(U.T @ U - np.eye(r)).max() <= tol and np.abs(Vt @ Vt.T - np.eye(r)).max() <= tol
     assert np.abs(S - np.linalg.svd(M, compute_uv=False)).max() <= tol * np.linalg.norm(M)
+
+
+# the same at scales whose squares leave FP64's range altogether, and through the kernel for what fits no cluster; the
+# rule has to keep the same rank
+@pytest.mark.parametrize("m,n", [(24, 16), (64, 40), (40, 64), (345, 340)])
+@pytest.mark.parametrize("scale", [1e200, 1e-200, 1e300, 1e-280])
+def test_svd_at_the_ends_of_the_range(m, n, scale):
+    rng = np.random.default_rng(m * 2000 + n)
+    r = min(m, n)
+    M = rng.standard_normal((m, r)) * 10.0 ** -np.linspace(0, 6, r) @ rng.standard_normal((r, n))
+    k0 = ttfit.tt_svd_truncated(M, chi_max=r, tau_rel=1e-3)[3]
+    U, S, Vt, k = ttfit.tt_svd_truncated(M * scale, chi_max=r, tau_rel=1e-3)
+    U, S, Vt = U.cpu().numpy(), S.cpu().numpy() / scale, Vt.cpu().numpy()
+    tol = 60 * r * EPS  # as above
+    assert k == k0
+    assert np.linalg.norm(U * S[None, :] @ Vt - M) <= tol * np.linalg.norm(M)
+    assert np.abs(U.T @ U - np.eye(r)).max() <= tol and np.abs(Vt @ Vt.T - np.eye(r)).max() <= tol
+
+
+@pytest.mark.parametrize("m,n", [(24, 16), (64, 40), (40, 64)])
+def test_svd_with_one_very_large_entry(m, n):
+    M = np.random.default_rng(0).standard_normal((m, n))
+    M[3, 5] = 1e200
+    U, S, Vt, k = ttfit.tt_svd_truncated(M, chi_max=min(m, n), tau_rel=0.0)
+    assert k == 1 and abs(float(S[0]) / 1e200 - 1) <= 60 * min(m, n) * EPS
+    assert bool(torch.isfinite(U).all() and torch.isfinite(S).all() and torch.isfinite(Vt).all())
+    assert abs(abs(float(U[3, 0])) - 1) <= 60 * min(m, n) * EPS and abs(abs(float(Vt[0, 5])) - 1) <= 60 * min(m, n) * EPS
+    M[:] = 1.7e308  # the largest singular value is not a number of FP64
+    with pytest.raises(ttfit.TTError) as e:
+        ttfit.tt_svd_truncated(M, chi_max=1, tau_rel=0.0)
+    assert e.value.code == ttfit.TT_ERR_NUMERICAL
