@@ -154,9 +154,16 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
   __shared__ int lifts[64], ups[64];
   if (l == 0) ups[grp] = 0;
   {
+    S x[RP][N];
     int f = 0;
-    if (c < p)
-      for (int i = l; i < q; i += LP) f = max(f, (__double2hiint(Xg[(size_t)c * q + i]) >> 20) & 0x7FF);
+#pragma unroll
+    for (int t = 0; t < RP; ++t)
+#pragma unroll
+      for (int h = 0; h < N; ++h) {
+        const int i = N * (l + LP * t) + h;
+        x[t][h] = (c < p && i < q) ? Xg[(size_t)c * q + i] : S(0);
+        f = max(f, (__double2hiint(x[t][h]) >> 20) & 0x7FF);
+      }
 #pragma unroll
     for (int o = LP / 2; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
     const int lift = A::lift(f, top);
@@ -164,10 +171,7 @@ __global__ void __launch_bounds__(RP == 16 ? 256 : 512)
 #pragma unroll
     for (int t = 0; t < RP; ++t)
 #pragma unroll
-      for (int h = 0; h < N; ++h) {
-        const int i = N * (l + LP * t) + h;
-        a[t].e[h] = (c < p && i < q) ? C(shift_bits(Xg[(size_t)c * q + i], lift)) : zero;
-      }
+      for (int h = 0; h < N; ++h) a[t].e[h] = C(shift_bits(x[t][h], lift));
   }
   auto publish = [&](int j) {  // my column (j) to every CTA, zeros above row j
     V* dst = pub + (j & 1) * LP * RP + l;
