@@ -290,7 +290,12 @@ __global__ void __launch_bounds__(1024)
   refresh();
   for (int w = threadIdx.x; w < 2 * b; w += blockDim.x) {
     const int sl = w / b, k = w % b;
-    nrm[w] = cid(cur, sl, k) >= 0 ? sqrt(col(cur, sl, k)[ld - 4]) : -1.0;
+    double v = cid(cur, sl, k) >= 0 ? sqrt(col(cur, sl, k)[ld - 4]) : -1.0;
+    if (!(v <= DBL_MAX)) {  // reported; and NaN would have no place in the order, so that outputs stayed unwritten
+      v = __longlong_as_double(0x7FF0000000000000ll);
+      if (errw) atomicOr(errw, ERRW_NAN);
+    }
+    nrm[w] = v;
   }
   cl.sync();
   for (int w = warp; w < 2 * b; w += nw) {  // every column's rank among all p (descending, ties by column index)

@@ -108,3 +108,13 @@ def test_svd_with_one_very_large_entry(m, n):
     with pytest.raises(ttfit.TTError) as e:
         ttfit.tt_svd_truncated(M, chi_max=1, tau_rel=0.0)
     assert e.value.code == ttfit.TT_ERR_NUMERICAL
+
+
+@pytest.mark.parametrize("m,n", [(24, 16), (40, 64), (120, 100)])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_svd_refuses_what_is_not_finite(m, n, value):
+    M = np.random.default_rng(0).standard_normal((m, n))
+    M[m // 2, n // 2] = value
+    with pytest.raises(ttfit.TTError) as e:
+        ttfit.tt_svd_truncated(M, chi_max=min(m, n), tau_rel=0.0)
+    assert e.value.code == ttfit.TT_ERR_NUMERICAL

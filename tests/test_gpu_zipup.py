@@ -222,3 +222,13 @@ def test_zipup_does_not_depend_on_the_scale(K, chi, e):
     A[-1] = A[-1] * 2.0 ** e
     C = ttfit.tt_mpo_zipup(A, B, chi, 0.0, **kw)
     assert torch.equal(C[0] * 2.0 ** -e, R[0]) and all(torch.equal(c, r) for c, r in zip(C[1:], R[1:]))
+
+
+@pytest.mark.parametrize("tol", [0.0, 1e-3])
+def test_zipup_refuses_a_gram_matrix_that_overflows(tol):
+    """Finite cores, finite M (1600 rows), but M^T M is not: no result rather than one made of it."""
+    A, B = (kron_sum_mpo(3, 40, 0, w) for w in (0, 1))
+    A[-1] = A[-1] * 2.0 ** 560
+    with pytest.raises(ttfit.TTError) as e:
+        ttfit.tt_mpo_zipup(A, B, 40, tol, update="svd", precision="fp64", prepare_inputs=0)
+    assert e.value.code == ttfit.TT_ERR_NUMERICAL
