@@ -353,7 +353,9 @@ tt_status tt_mpo_grad(const tt_mpo_desc* A, const tt_mpo_desc* B, const tt_mpo_d
  * into caller device buffers U (m x r row-major), S (r), Vt (r x n
  * row-major), r = min(m, n) <= 1024, and returns in *k_out (host) the rank
  * the truncation rule keeps: k = min(chi_max, min{k : sqrt(sum_{j>k} s_j^2)
- * <= tau_rel ||M||_F}), values <= 1e-13 s_1 dropped, k >= 1. Takes its
+ * <= tau_rel ||M||_F}), values <= 1e-13 s_1 dropped, k >= 1. The r x r factor
+ * is orthogonal whatever the rank; in the other one the columns of values that
+ * are null, or rounding of null, may be zero or not orthogonal. Takes its
  * scratch from the block cache (tt_device_cache_release), runs on `stream`
  * (cudaStream_t, NULL = default) and synchronises it. Errors: TT_ERR_INVALID_ARGUMENT (NULL pointer,
  * non-positive size, r > 1024), TT_ERR_OUT_OF_MEMORY, TT_ERR_CUDA,

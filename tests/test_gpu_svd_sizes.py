@@ -118,3 +118,30 @@ def test_svd_refuses_what_is_not_finite(m, n, value):
     with pytest.raises(ttfit.TTError) as e:
         ttfit.tt_svd_truncated(M, chi_max=min(m, n), tau_rel=0.0)
     assert e.value.code == ttfit.TT_ERR_NUMERICAL
+
+
+# null columns, null rows, equal columns, the null matrix; one CTA and clusters, the long side on either hand
+@pytest.mark.parametrize("m,n", [(24, 16), (33, 32), (64, 40), (40, 64), (130, 120)])
+@pytest.mark.parametrize("kind", ["columns", "rows", "rank1", "zero"])
+def test_svd_of_a_rank_deficient_matrix(m, n, kind):
+    r = min(m, n)
+    M = np.random.default_rng(m).standard_normal((m, n))
+    if kind == "columns":
+        M[:, n // 2:] = 0.0
+    elif kind == "rows":
+        M[m // 2:] = 0.0
+    elif kind == "rank1":
+        M[:] = 1.0
+    else:
+        M[:] = 0.0
+    U, S, Vt, k = ttfit.tt_svd_truncated(M, chi_max=r, tau_rel=0.0)
+    U, S, Vt = U.cpu().numpy(), S.cpu().numpy(), Vt.cpu().numpy()
+    tol = 60 * r * EPS  # as above
+    rank = np.linalg.matrix_rank(M)
+    assert k == max(rank, 1)
+    assert np.linalg.norm(U * S[None, :] @ Vt - M) <= tol * np.linalg.norm(M)
+    assert np.abs(S - np.linalg.svd(M, compute_uv=False)).max() <= tol * np.linalg.norm(M)
+    square = Vt if m >= n else U.T  # the r x r factor is orthogonal whatever the rank
+    assert np.abs(square @ square.T - np.eye(r)).max() <= tol
+    long = U[:, :rank] if m >= n else Vt[:rank].T
+    assert np.abs(long.T @ long - np.eye(rank)).max(initial=0.0) <= tol
