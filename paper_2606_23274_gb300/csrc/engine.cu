@@ -109,6 +109,7 @@ struct BlockCache {
     std::vector<std::pair<std::pair<int, size_t>, void*>> drop;
     {
       std::lock_guard<std::mutex> g(mu);
+      drop.reserve(free_blocks.size());  // nothing throws from here on
       for (size_t i = 0; i < free_blocks.size();)
         if (dev < 0 || free_blocks[i].first.first == dev) {
           drop.push_back(free_blocks[i]);
@@ -142,20 +143,31 @@ BlockCache& block_cache() {
 
 namespace ttfit {
 
-void* block_take(int dev, size_t bytes, size_t* got) {
+// Neither throws: they are called from C entry points and destructors, and the cache's own lists may find no host memory.
+void* block_take(int dev, size_t bytes, size_t* got) noexcept {
   bytes = (std::max<size_t>(bytes, 1) + 511) & ~(size_t)511;
   *got = bytes;
-  void* p = block_cache().take(dev, bytes, got);
-  if (p) return p;
-  if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
-  cudaGetLastError();
-  block_cache().trim(dev);
+  void* p = nullptr;
+  try {
+    p = block_cache().take(dev, bytes, got);
+    if (p) return p;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    block_cache().trim(dev);
+  } catch (...) {
+  }
   if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
   cudaGetLastError();
   return nullptr;
 }
 
-void block_give(int dev, size_t bytes, void* p) { block_cache().give(dev, bytes, p); }
+void block_give(int dev, size_t bytes, void* p) noexcept {
+  try {
+    block_cache().give(dev, bytes, p);
+  } catch (...) {  // not kept: nothing after the last insertion throws
+    cudaFree(p);
+  }
+}
 
 }  // namespace ttfit
 
@@ -184,13 +196,13 @@ struct DevPool {
   void release(void* p) {
     for (auto& b : blks)
       if (b.p == p) {
-        block_cache().give(b.dev, b.bytes, b.p);
+        block_give(b.dev, b.bytes, b.p);
         b.p = nullptr;
       }
   }
   ~DevPool() {
     for (auto& b : blks)
-      if (b.p) block_cache().give(b.dev, b.bytes, b.p);
+      if (b.p) block_give(b.dev, b.bytes, b.p);
   }
 };
 
@@ -3092,7 +3104,13 @@ tt_status tt_fit_launch_count(const tt_fit* h, long long* n) {
   return TT_OK;
 }
 
-size_t tt_device_cache_release(int device) { return block_cache().trim(device); }
+size_t tt_device_cache_release(int device) {
+  try {
+    return block_cache().trim(device);
+  } catch (...) {  // no host memory for the list: nothing was freed
+    return 0;
+  }
+}
 
 tt_status tt_fit_jacobi_sweeps(const tt_fit* h, int* max_sweeps) {
   if (!h || !max_sweeps) return TT_ERR_INVALID_ARGUMENT;

@@ -59,15 +59,16 @@ struct Arena {
   explicit Arena(cudaStream_t s) : st(s) { cudaGetDevice(&dev); }
   template <typename T>
   T* alloc(size_t n) {
-    size_t got = 0;
-    void* p = block_take(dev, std::max<size_t>(n, 1) * sizeof(T), &got);
-    if (!p) throw GradError(TT_ERR_OUT_OF_MEMORY, "cudaMalloc of " + std::to_string(n * sizeof(T)) + " bytes failed");
-    blks.push_back({p, got});
-    return (T*)p;
+    blks.push_back({nullptr, 0});  // its place first: nothing throws while a block is in hand
+    Blk& b = blks.back();
+    b.p = block_take(dev, std::max<size_t>(n, 1) * sizeof(T), &b.bytes);
+    if (!b.p) throw GradError(TT_ERR_OUT_OF_MEMORY, "cudaMalloc of " + std::to_string(n * sizeof(T)) + " bytes failed");
+    return (T*)b.p;
   }
   ~Arena() {
     if (!blks.empty()) cudaStreamSynchronize(st);
-    for (auto& b : blks) block_give(dev, b.bytes, b.p);
+    for (auto& b : blks)
+      if (b.p) block_give(dev, b.bytes, b.p);
   }
   Arena(const Arena&) = delete;
   Arena& operator=(const Arena&) = delete;

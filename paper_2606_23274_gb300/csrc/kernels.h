@@ -9,8 +9,8 @@ namespace ttfit {
 // The process-wide cache of device blocks (engine.cu): a block of at least `bytes` on the current device dev
 // (*got: its size, to be handed back with it), null when the device has no room. A block is given back only after
 // the streams that used it have been synchronised.
-void* block_take(int dev, size_t bytes, size_t* got);
-void block_give(int dev, size_t bytes, void* p);
+void* block_take(int dev, size_t bytes, size_t* got) noexcept;
+void block_give(int dev, size_t bytes, void* p) noexcept;
 
 template <typename T>
 struct GemmArgs {
