@@ -15,44 +15,38 @@ namespace ttfit {
 // cluster), with one column of a pair kept in registers while it meets its partners, and |w|^2 carried along. A pair's
 // micro-round is a chain of about 500 cycles (loads, dot product, butterfly, angle, update); 138 columns take 64 us a
 // sweep on 8 CTAs, 75 on 4; 74 columns 31 on 4, 35 on 8.
-// One pair of FP32 columns with the rows of x in registers (kept by the caller), those of y loaded and stored.
-template <int LP, int NV>
+// One pair of FP32 columns, worked by a warp, with the rows of x in registers (kept by the caller), those of y loaded
+// and stored.
+template <int NV>
 struct Col32 {
   float4 v[NV];
 };
 
-template <int LP>
-__device__ __forceinline__ float lanes_sum32(float v) {
-#pragma unroll
-  for (int o = LP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 constexpr int J32_TAIL = 4;  // trailer of a column: |w|^2
 
-template <int LP, int NV>
-__device__ __forceinline__ bool jacobi32_pair(Col32<LP, NV>& x, float& a, float* __restrict__ xj, int nq, int nr, int ld,
+template <int NV>
+__device__ __forceinline__ bool jacobi32_pair(Col32<NV>& x, float& a, float* __restrict__ xj, int nq, int nr, int ld,
                                               float tol, bool act) {
-  const int l = threadIdx.x & (LP - 1);
+  const int l = threadIdx.x & 31;
   float4* y4 = reinterpret_cast<float4*>(xj);
-  Col32<LP, NV> y;
+  Col32<NV> y;
   float g0 = 0.f, g1 = 0.f;
   const float b = xj[ld - J32_TAIL];
 #pragma unroll
   for (int t = 0; t < NV; ++t) {
-    const int r = l + LP * t;
+    const int r = l + 32 * t;
     if (r < nr) y.v[t] = y4[r];
     else y.v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
 #pragma unroll
   for (int t = 0; t < NV; ++t)
-    if (l + LP * t < nq) {
+    if (l + 32 * t < nq) {
       g0 = fmaf(x.v[t].x, y.v[t].x, g0);
       g1 = fmaf(x.v[t].y, y.v[t].y, g1);
       g0 = fmaf(x.v[t].z, y.v[t].z, g0);
       g1 = fmaf(x.v[t].w, y.v[t].w, g1);
     }
-  const float g = lanes_sum32<LP>(g0 + g1);
+  const float g = warp_sum(g0 + g1);
   // the cosine itself: squares of small columns' products would underflow; columns below 1e-16 of the largest stay
   const bool rot = act && a > 1e-32f && b > 1e-32f && fabsf(g) * rsqrtf(a) * rsqrtf(b) > tol;
   __syncwarp();  // every lane has read the trailers, which lane 0 is about to replace (a shuffle orders no memory)
@@ -68,7 +62,7 @@ __device__ __forceinline__ bool jacobi32_pair(Col32<LP, NV>& x, float& a, float*
       const float4 u = x.v[k], w = y.v[k];
       x.v[k] = make_float4(fmaf(cs, u.x, -sn * w.x), fmaf(cs, u.y, -sn * w.y), fmaf(cs, u.z, -sn * w.z), fmaf(cs, u.w, -sn * w.w));
       const float4 z = make_float4(fmaf(cs, w.x, sn * u.x), fmaf(cs, w.y, sn * u.y), fmaf(cs, w.z, sn * u.z), fmaf(cs, w.w, sn * u.w));
-      if (l + LP * k < nr) y4[l + LP * k] = z;
+      if (l + 32 * k < nr) y4[l + 32 * k] = z;
     }
     a = fmaf(-t, g, a);
     if (l == 0) xj[ld - J32_TAIL] = fmaf(t, g, b);
@@ -76,26 +70,26 @@ __device__ __forceinline__ bool jacobi32_pair(Col32<LP, NV>& x, float& a, float*
   return rot;
 }
 
-template <int LP, int NV>
-__device__ __forceinline__ void load32(Col32<LP, NV>& x, const float* p, int nr) {
-  const int l = threadIdx.x & (LP - 1);
+template <int NV>
+__device__ __forceinline__ void load32(Col32<NV>& x, const float* p, int nr) {
+  const int l = threadIdx.x & 31;
 #pragma unroll
   for (int t = 0; t < NV; ++t)
-    x.v[t] = l + LP * t < nr ? reinterpret_cast<const float4*>(p)[l + LP * t] : make_float4(0.f, 0.f, 0.f, 0.f);
+    x.v[t] = l + 32 * t < nr ? reinterpret_cast<const float4*>(p)[l + 32 * t] : make_float4(0.f, 0.f, 0.f, 0.f);
 }
-template <int LP, int NV>
-__device__ __forceinline__ void store32(const Col32<LP, NV>& x, float* p, int nr) {
-  const int l = threadIdx.x & (LP - 1);
+template <int NV>
+__device__ __forceinline__ void store32(const Col32<NV>& x, float* p, int nr) {
+  const int l = threadIdx.x & 31;
 #pragma unroll
   for (int t = 0; t < NV; ++t)
-    if (l + LP * t < nr) reinterpret_cast<float4*>(p)[l + LP * t] = x.v[t];
+    if (l + 32 * t < nr) reinterpret_cast<float4*>(p)[l + 32 * t] = x.v[t];
 }
 
 __host__ __device__ inline int jacobi32_ld(int q, int p) {
   return (q + 3) / 4 * 4 + (p + 3) / 4 * 4 + J32_TAIL;
 }
 
-template <int LP, int NV>
+template <int NV>
 __global__ void __launch_bounds__(640)
     jacobi32_kernel(int q, int p, int b, const float* __restrict__ Win, int max_sweeps, float ftol,
                     float* __restrict__ Vo) {
@@ -105,15 +99,12 @@ __global__ void __launch_bounds__(640)
   const int qs = (q + 3) / 4 * 4;
   const int ld = jacobi32_ld(q, p);
   const int nq = qs / 4, nr = (ld - J32_TAIL) / 4;
-  const int nbuf = NC > 1 ? 2 : 1;
   extern __shared__ __align__(16) unsigned char j32s[];
-  float* buf = (float*)j32s;                                  // [nbuf][2 slots][b][ld]
-  int* ids = (int*)(buf + (size_t)nbuf * 2 * b * ld);         // [nbuf][2 slots][b] global column or -1
+  float* buf = (float*)j32s;                                  // [2][2 slots][b][ld]
+  int* ids = (int*)(buf + (size_t)4 * b * ld);                // [2][2 slots][b] global column or -1
   float* nrm = (float*)(ids + 4 * b + 4);                     // [2 slots][b] final column norms
   __shared__ int flag[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  constexpr int G = 32 / LP;
-  const int grp = warp * G + lane / LP, ng = nw * G, l = lane & (LP - 1);
   auto col = [&](int bi, int sl, int k) { return buf + ((size_t)(bi * 2 + sl) * b + k) * ld; };
   auto cid = [&](int bi, int sl, int k) -> int& { return ids[(bi * 2 + sl) * b + k]; };
 
@@ -135,24 +126,24 @@ __global__ void __launch_bounds__(640)
 
   int cur = 0, sweep = 0;
   auto refresh = [&]() {  // |w|^2 of every column, from its rows
-    for (int w0 = 0; w0 < 2 * b; w0 += ng) {
-      const int w = w0 + grp;
+    for (int w0 = 0; w0 < 2 * b; w0 += nw) {
+      const int w = w0 + warp;
       float s = 0.f;
       float* x = col(cur, w < b ? 0 : 1, w < 2 * b ? w % b : 0);
       if (w < 2 * b) {
         const float4* x4 = reinterpret_cast<const float4*>(x);
-        for (int r = l; r < nq; r += LP) {
+        for (int r = lane; r < nq; r += 32) {
           const float4 v = x4[r];
           s = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s))));
         }
       }
-      s = lanes_sum32<LP>(s);
-      if (w < 2 * b && l == 0) x[ld - J32_TAIL] = s;
+      s = warp_sum(s);
+      if (w < 2 * b && lane == 0) x[ld - J32_TAIL] = s;
     }
     __syncthreads();
   };
   bool done = false;
-  Col32<LP, NV> x;
+  Col32<NV> x;
   while (!done && sweep < max_sweeps) {
     bool rot = false;
     refresh();
@@ -160,44 +151,40 @@ __global__ void __launch_bounds__(640)
       if (sr == 0) {  // pairs inside each block (round robin over the b columns of both slots)
         const int B = b + (b & 1), half = B / 2;
         for (int mr = 0; mr < B - 1; ++mr) {
-          const int sl = grp / half, k = grp % half;
+          const int sl = warp / half, k = warp % half;
           int i = b, j = b;
-          if (grp < 2 * half) rr_pair(mr, k, B, i, j);
+          if (warp < 2 * half) rr_pair(mr, k, B, i, j);
           const bool act = i < b && j < b;
           float* xi = col(cur, act ? sl : 0, act ? i : 0);
           float a = xi[ld - J32_TAIL];
           load32(x, xi, act ? nr : 0);
-          const bool r1 = jacobi32_pair<LP, NV>(x, a, col(cur, act ? sl : 0, act ? j : 0), nq, nr, ld, ftol, act);
+          const bool r1 = jacobi32_pair<NV>(x, a, col(cur, act ? sl : 0, act ? j : 0), nq, nr, ld, ftol, act);
           if (r1) {
             store32(x, xi, nr);
-            if (l == 0) xi[ld - J32_TAIL] = a;
+            if (lane == 0) xi[ld - J32_TAIL] = a;
           }
           rot |= r1;
           __syncthreads();
         }
       }
-      {  // pairs between the two blocks: group w keeps column w of slot 0 in registers and meets column
+      {  // pairs between the two blocks: warp w keeps column w of slot 0 in registers and meets column
          // (w + mr) mod b of slot 1
-        const bool act = grp < b;
-        float* xi = col(cur, 0, act ? grp : 0);
+        const bool act = warp < b;
+        float* xi = col(cur, 0, act ? warp : 0);
         float a = xi[ld - J32_TAIL];
         load32(x, xi, act ? nr : 0);
         bool changed = false;
-        int j = act ? grp : 0;
+        int j = act ? warp : 0;
         for (int mr = 0; mr < b; ++mr) {
-          changed |= jacobi32_pair<LP, NV>(x, a, col(cur, 1, j), nq, nr, ld, ftol, act);
+          changed |= jacobi32_pair<NV>(x, a, col(cur, 1, j), nq, nr, ld, ftol, act);
           j = (j + 1 == b) ? 0 : j + 1;
           __syncthreads();
         }
         if (changed) {
           store32(x, xi, nr);
-          if (l == 0) xi[ld - J32_TAIL] = a;
+          if (lane == 0) xi[ld - J32_TAIL] = a;
         }
         rot |= changed;
-      }
-      if (NC == 1) {
-        __syncthreads();
-        break;  // two blocks: one super-round
       }
       // rotate the positions 1..P-1 by one (position 0 stays): pull the next two blocks
       cl.sync();
@@ -278,8 +265,8 @@ __global__ void __launch_bounds__(640)
 }
 
 inline size_t jacobi32_smem(int q, int p, int nc) {
-  const size_t b = (p + 2 * nc - 1) / (2 * nc), nbuf = nc > 1 ? 2 : 1;
-  return nbuf * 2 * b * jacobi32_ld(q, p) * sizeof(float) + (4 * b + 4) * sizeof(int) + 2 * b * sizeof(float) + 16;
+  const size_t b = (p + 2 * nc - 1) / (2 * nc);
+  return 4 * b * jacobi32_ld(q, p) * sizeof(float) + (4 * b + 4) * sizeof(int) + 2 * b * sizeof(float) + 16;
 }
 
 namespace {
@@ -328,11 +315,11 @@ cudaError_t jacobi32_rotations(int p, const float* W, float* V, int sweeps, cuda
     return e != cudaSuccess ? e : cudaGetLastError();
   };
   switch (s.nv) {
-    case 1: return launch(jacobi32_kernel<32, 1>);
-    case 2: return launch(jacobi32_kernel<32, 2>);
-    case 3: return launch(jacobi32_kernel<32, 3>);
-    case 4: return launch(jacobi32_kernel<32, 4>);
-    default: return launch(jacobi32_kernel<32, 5>);
+    case 1: return launch(jacobi32_kernel<1>);
+    case 2: return launch(jacobi32_kernel<2>);
+    case 3: return launch(jacobi32_kernel<3>);
+    case 4: return launch(jacobi32_kernel<4>);
+    default: return launch(jacobi32_kernel<5>);
   }
 }
 

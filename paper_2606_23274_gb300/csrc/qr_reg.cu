@@ -347,10 +347,10 @@ cudaError_t qr_reg_launch(int nc, int lp, int q, int p, int top, S* X, S* Q, S* 
   const int threads = ((p + nc - 1) / nc * lp + 31) / 32 * 32;
   const int rp = q <= 4 * N * lp ? 4 : q <= 8 * N * lp ? 8 : 16;
   if (threads > (rp == 16 ? 256 : 512) || q > 16 * N * lp) return cudaErrorNotSupported;
-  const size_t sm = (size_t)2 * lp * rp * 16 + 2 * (size_t)std::min(q, p) * sizeof(C);
+  if (lp < 32 && rp != 4) return cudaErrorNotSupported;  // the callers take 32 lanes for such columns
+  const size_t sm = (size_t)2 * lp * rp * 16 + 2 * (size_t)std::min(q, p) * sizeof(C);  // 20 KB at most
   auto launch = [&](auto kern) -> cudaError_t {
     cudaError_t e;
-    if (sm > 48 * 1024 && (e = ensure_smem((const void*)kern, sm)) != cudaSuccess) return e;
     if (nc > 8 &&
         (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
       return e;
@@ -377,10 +377,9 @@ cudaError_t qr_reg_launch(int nc, int lp, int q, int p, int top, S* X, S* Q, S* 
     e = cudaLaunchKernelEx(&cfg, kern, q, p, top, X, Q, R);
     return e != cudaSuccess ? e : cudaGetLastError();
   };
-  if (lp == 8)
-    return rp == 4 ? launch(qr_reg_kernel<S, C, 8, 4>) : rp == 8 ? launch(qr_reg_kernel<S, C, 8, 8>) : launch(qr_reg_kernel<S, C, 8, 16>);
-  if (lp == 16)
-    return rp == 4 ? launch(qr_reg_kernel<S, C, 16, 4>) : rp == 8 ? launch(qr_reg_kernel<S, C, 16, 8>) : launch(qr_reg_kernel<S, C, 16, 16>);
+  if constexpr (std::is_same<C, double>::value)
+    if (lp == 8) return launch(qr_reg_kernel<S, C, 8, 4>);
+  if (lp == 16) return launch(qr_reg_kernel<S, C, 16, 4>);
   return rp == 4 ? launch(qr_reg_kernel<S, C, 32, 4>) : rp == 8 ? launch(qr_reg_kernel<S, C, 32, 8>) : launch(qr_reg_kernel<S, C, 32, 16>);
 }
 
