@@ -133,7 +133,7 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = svd_tall64(q, r, X, Ux, Vw, extra, extra ? extra + (size_t)r * r : nullptr, &Ux, Sv, Vx, 60, info, sms, st)) != cudaSuccess) return e;
-  if (r >= 32) {  // below, V is the product of the rotations
+  if (Ux == X) {  // by way of the QR; else V is the product of the rotations
     ++tl_launches;
     complete_basis_kernel<<<1, 1024, 0, st>>>(r, Vx, Sv);
   }
