@@ -2,8 +2,8 @@
 //
 //   C[cm(m) + cn(n)] = alpha * sum_k A[m*lda + k] * B(n, k) + beta * C[...]
 //
-// A is K-major (k contiguous, rows at stride lda); B is K-major (rows n at
-// stride ldb, k contiguous) or MN-major (rows k at stride ldb, n contiguous).
+// A is K-major (k contiguous, rows at stride lda), and so is B (rows n at
+// stride ldb).
 // Operand tiles are moved global -> shared memory by TMA (128-byte swizzle),
 // one elected thread issues tcgen05.mma (kind::tf32, FP32 accumulation in
 // tensor memory), and four warps drain the 128 x 128 accumulator with
@@ -105,10 +105,9 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 
 // instruction descriptor: D = F32 (bits 4-5 = 1), A = B = TF32 (format 2 at bits 7-9 and 10-12),
-// A K-major (bit 15 = 0), B major per template (bit 16), N >> 3 at bits 17-22, M >> 4 at bits 24-28
-__host__ __device__ constexpr uint32_t idesc_tf32(int m, int n, bool b_mn_major) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(m >> 4) << 24);
+// both K-major (bits 15 and 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28
+__host__ __device__ constexpr uint32_t idesc_tf32(int m, int n) {
+  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 // kind::f16 with both operands BF16 (format 1 at bits 7-9 and 10-12), D = F32, both K-major
@@ -124,7 +123,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-template <bool B_MN, bool SPLIT, bool OVERLAP>
+template <bool SPLIT, bool OVERLAP>
 __global__ void __launch_bounds__(128, OVERLAP ? 3 : 1)
     gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N,
                      int K, int k_per_split, float* __restrict__ C, IdxMap cm, IdxMap cn, float alpha, float beta,
@@ -183,18 +182,12 @@ __global__ void __launch_bounds__(128, OVERLAP ? 3 : 1)
       mbar_expect_tx(full, 2 * TILE_BYTES);
       const int k = kb0 + kb * BK;
       tma_load_2d(su32(sA + s * TILE_BYTES), &tmA, full, k, m0);
-      if (B_MN) {
-        // four boxes of (32 n) x (BK k): n chunk j at byte offset j * BK * 128
-#pragma unroll
-        for (int j = 0; j < BN / 32; ++j) tma_load_2d(su32(sB + s * TILE_BYTES + j * BK * 128), &tmB, full, n0 + 32 * j, k);
-      } else {
-        tma_load_2d(su32(sB + s * TILE_BYTES), &tmB, full, k, n0);
-      }
+      tma_load_2d(su32(sB + s * TILE_BYTES), &tmB, full, k, n0);
       issued = kb + 1;
     }
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer
-    const uint32_t idesc = idesc_tf32(BM, BN, B_MN);
+    const uint32_t idesc = idesc_tf32(BM, BN);
     bool ok = true;
     for (int kb = 0; kb < nk; ++kb) {
       const int s = kb % STAGES;
@@ -212,9 +205,7 @@ __global__ void __launch_bounds__(128, OVERLAP ? 3 : 1)
       for (int kk = 0; kk < BK / 8; ++kk) {
         // K-major: advance 8 tf32 = 32 bytes inside the swizzle span; SBO = 8 rows x 128 B
         const uint64_t ad = sdesc(a_base + kk * 32, 16, 1024);
-        uint64_t bd;
-        if (B_MN) bd = sdesc(b_base + kk * 1024, BK * 128, 1024);  // 8 k-rows per step; LBO = n-chunk stride
-        else bd = sdesc(b_base + kk * 32, 16, 1024);
+        const uint64_t bd = sdesc(b_base + kk * 32, 16, 1024);
         mma_tf32(tmem, ad, bd, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
         if (SPLIT) {  // + A_hi B_lo + A_lo B_hi (the tensor core truncates A, B to their TF32 high parts)
           const uint64_t bdl = sdesc(su32(sBl + s * TILE_BYTES) + kk * 32, 16, 1024);
@@ -510,7 +501,7 @@ __device__ __forceinline__ void oz_mma(uint32_t tmem, uint64_t ad, uint64_t bd, 
   if constexpr (sizeof(D) == 2)
     mma_bf16(tmem, ad, bd, idesc_bf16(BM, BN), acc ? 1u : 0u);
   else
-    mma_tf32(tmem, ad, bd, idesc_tf32(BM, BN, false), acc ? 1u : 0u);
+    mma_tf32(tmem, ad, bd, idesc_tf32(BM, BN), acc ? 1u : 0u);
 }
 
 // One 128 x 128 output tile of one K-chunk (blockIdx.z) into the double-FP32
@@ -675,19 +666,14 @@ cudaError_t gemm_tf32(const GemmArgs<float>& g, float* ws, size_t ws_elems, int 
   if (!lin_stride(g.am, lda) || !lin_stride(g.ak, one) || one != 1) return cudaErrorNotSupported;
   // B must be K-major: an MN-major B with kind::tf32 produced an all-zero
   // accumulator in the self-check, so such layouts go to the CUDA-core kernel.
-  bool b_mn = false;
   if (!(lin_stride(g.bk, one) && one == 1 && lin_stride(g.bn, ldb))) return cudaErrorNotSupported;
   // TMA: 16-byte aligned bases and row strides
   if (((uintptr_t)g.A & 15) || ((uintptr_t)g.B & 15) || (lda * 4) % 16 || (ldb * 4) % 16) return cudaErrorNotSupported;
-  if (lda < g.K || (!b_mn && ldb < g.K) || (b_mn && ldb < g.N)) return cudaErrorNotSupported;
+  if (lda < g.K || ldb < g.K) return cudaErrorNotSupported;
   if (g.K < 1) return cudaErrorNotSupported;
   CUtensorMap ta, tb;
   if (!make_map(&ta, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)lda, BK, BM)) return cudaErrorNotSupported;
-  if (!b_mn) {
-    if (!make_map(&tb, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)ldb, BK, BN)) return cudaErrorNotSupported;
-  } else {
-    if (!make_map(&tb, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)ldb, 32, BK)) return cudaErrorNotSupported;
-  }
+  if (!make_map(&tb, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)ldb, BK, BN)) return cudaErrorNotSupported;
   const int gm = (g.M + BM - 1) / BM, gn = (g.N + BN - 1) / BN;
   int splits = 1;
   while (gm * gn * splits < sm_count && g.K / (splits * 2) >= 4 * BK && (size_t)(splits * 2) * g.M * g.N <= ws_elems)
@@ -707,9 +693,9 @@ cudaError_t gemm_tf32(const GemmArgs<float>& g, float* ws, size_t ws_elems, int 
   };
   cudaError_t e;
   if (split && (long long)gm * gn * splits >= 2 * sm_count)
-    e = launch(gemm_tf32_kernel<false, true, true>, Cfg<true, true>::SMEM_BYTES);
-  else if (split) e = launch(gemm_tf32_kernel<false, true, false>, Cfg<true>::SMEM_BYTES);
-  else e = launch(gemm_tf32_kernel<false, false, false>, Cfg<false>::SMEM_BYTES);
+    e = launch(gemm_tf32_kernel<true, true>, Cfg<true, true>::SMEM_BYTES);
+  else if (split) e = launch(gemm_tf32_kernel<true, false>, Cfg<true>::SMEM_BYTES);
+  else e = launch(gemm_tf32_kernel<false, false>, Cfg<false>::SMEM_BYTES);
   if (e != cudaSuccess || splits == 1) return e;
   return splitk_reduce<float>(g, ws, splits, sm_count, st);
 }
