@@ -15,7 +15,7 @@ namespace ttfit {
 constexpr int BK = 16, NT = 256;
 
 // Tile edge TB = 16 MT: a 16 x 16 thread grid, MT x MT outputs a thread. FP64 and df32 tiles are bound
-// by their SM's arithmetic (an FP64 multiply-add of a warp takes 19 cycles of an SM, a df32 one 15
+// by their SM's arithmetic (an FP64 multiply-add of a warp takes 17 cycles of an SM, a df32 one 15
 // FP32 instructions), so a small product is cut into small tiles, which spread over more SMs and carry
 // less padding; a tile's operand traffic stays far below what an SM can load in that time.
 template <typename T, int MT>

@@ -14,7 +14,7 @@ namespace ttfit {
 // ---------------------------------------------------------------------------
 // One-sided Jacobi in FP64 (cluster of 1, 8 or 16 CTAs), organised around the
 // FP64 pipe: a warp-wide FP64 instruction occupies its SM quadrant for 64 cycles
-// whatever number of lanes is active (measured; an SM issues one per 19 cycles),
+// whatever number of lanes is active (measured; an SM issues one per 17 cycles),
 // so what counts is the number of warp instructions, not of operations.
 //  * A column pair is worked by LP lanes, and a warp holds 32 / LP pairs: the
 //    butterfly of the dot product and the rotation angle, which every lane of a
@@ -410,7 +410,7 @@ cudaError_t jacobi_svd64(int q, int p, const double* W, const double* Vin, doubl
 }
 
 // SVD of a p x p matrix with graded columns, L = U diag(S) W^T.
-// Four fifths of the sweeps run in FP32, where they cost a quarter: an FP32 Jacobi of L gives rotations W0, made
+// The first sweeps, eight at most, run in FP32, where they cost a quarter: an FP32 Jacobi of L gives rotations W0, made
 // orthonormal to FP64 rounding by two Newton-Schulz steps, and the FP64 Jacobi of L W0 needs 3 or 4 sweeps for its own
 // stopping rule instead of 10 (spectra down to 1e-18 s_1: the columns are graded, so FP32 keeps each to its own
 // rounding). The result is as accurate as without: every rotation that counts is taken in FP64.
