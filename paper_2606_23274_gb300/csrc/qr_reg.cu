@@ -386,7 +386,7 @@ cudaError_t qr_reg_launch(int nc, int lp, int q, int p, int top, S* X, S* Q, S* 
 // FP64. CTAs and lanes a column by the measured times (us, with Q; the blocked cluster kernel or, for the
 // rows marked *, the one-CTA kernel takes): 64 x 20 *298: 4 CTAs of 8 lanes 72; 64 x 64 *1203: 8 x 8 209;
 // 100 x 37 *620: 8 x 16 138; 128 x 128 1397: 8 x 16 630; 256 x 74 934: 8 x 16 444, 16 x 32 328;
-// 512 x 128 2312: 8 x 16 1825, 16 x 32 1088.
+// 512 x 128 2312: 8 x 16 1825, 16 x 32 1095.
 cudaError_t qr_reg64(int q, int p, double* X, double* Q, double* R, cudaStream_t st, bool any_scale) {
   const int top = any_scale ? 1023 + 300 : 0x7FE;
   const int lp = q <= 64 ? 8 : q <= 128 ? 16 : 32;
@@ -398,7 +398,7 @@ cudaError_t qr_reg64(int q, int p, double* X, double* Q, double* R, cudaStream_t
 }
 
 // Double-FP32 arithmetic on FP64 storage. 128 x 128: 888 us by the blocked kernel, 284 here (8 CTAs of
-// 16 lanes); 256 x 64: 420, 169 (8 x 32); 512 x 128: 1199, 666 (8 x 32). Clusters of 16 take 578 for the
+// 16 lanes); 256 x 64: 420, 165 (8 x 32); 512 x 128: 1199, 628 (8 x 32). Clusters of 16 take 578 for the
 // last, but two chains and the random guess prepare at once, and 8 leave them room.
 cudaError_t qr_reg_df32(int q, int p, double* X, double* Q, double* R, cudaStream_t st) {
   return qr_reg_launch<double, df32>(8, q <= 128 ? 16 : 32, q, p, 0, X, Q, R, st);
