@@ -21,14 +21,15 @@ size_t svd_scratch_doubles(int m, int n) {
   const size_t r = std::min(m, n), q = std::max(m, n);
   return 2 * q * r + 2 * r * r + r + 1 + 2 + 2 + 1;
 }
-size_t svd_info_offset(int m, int n) {
-  const size_t r = std::min(m, n), q = std::max(m, n);
-  return 2 * q * r + 2 * r * r + r + 3;
-}
+
+// Columns of the square factor whose value is null, and what rounding left of them: where it is the left factor of R^T
+// (svd_tall64) they are zero, or not orthogonal. Below 2^-200 s_1 the squares of two columns' products vanish in the
+// Jacobi.
+__device__ __forceinline__ bool svd_null(const double* S, int j) { return !(S[j] > 0x1p-200 * S[0]); }
 
 __global__ void svd_outputs_kernel(int m, int n, int tr, const double* __restrict__ Ux, const double* __restrict__ Vx,
                                    const double* __restrict__ Sv, double* __restrict__ U, double* __restrict__ S,
-                                   double* __restrict__ Vt, uint32_t* errw) {
+                                   double* __restrict__ Vt, uint32_t* errw, uint32_t* nulls) {
   // X = Ux diag(S) Vx^T with X = M (tr = 0, Ux m x r) or X = M^T (tr = 1, Ux n x r)
   const int r = min(m, n);
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -44,71 +45,24 @@ __global__ void svd_outputs_kernel(int m, int n, int tr, const double* __restric
   for (long long e = t0; e < r; e += stride) {
     S[e] = Sv[e];
     if (!isfinite(Sv[e])) atomicOr(errw, ERRW_NAN);
+    if (nulls && svd_null(Sv, (int)e)) *nulls = 1;
   }
 }
 
-// Columns of V (p x p, column-major, p <= 1024) whose value is null: where V is the left factor of R^T (svd_tall64) they
-// are zero, or what rounding left. Here they become the rest of an orthonormal basis: the column itself, or, where that
-// is no new direction, the unit vector that the columns before it cover least (1/p of its square is left at least), less
-// its part in those columns, taken away twice. One CTA; returns at once where no value is null (256 x 256: 7.86 ms a call
-// before, 7.87 so; of rank 128, 7.2 and 15.9: three passes of FP64 operations a column on one SM).
-__global__ void __launch_bounds__(1024) complete_basis_kernel(int p, double* V, const double* S) {
-  __shared__ double w[1024], cf[1024];
-  __shared__ unsigned long long best;
-  const int i = threadIdx.x, warp = i >> 5, lane = i & 31;
-  const double lim = 0x1p-200 * S[0];  // below it the squares of two columns' products vanish in the Jacobi
-  const int k0 = __syncthreads_count(i < p && S[min(i, p - 1)] > lim);
-  double left = 1.0;  // of the square of unit vector i
-  if (i < p)
-    for (int k = 0; k < k0 && k0 < p; ++k) left = fma(-V[(size_t)k * p + i], V[(size_t)k * p + i], left);
-  for (int j = k0; j < p; ++j) {
-    double nrm = 0.0;
-    for (int attempt = S[j] > 0.0 ? 0 : 1; attempt < 2 && !(nrm > 0.5); ++attempt) {
-      if (attempt == 1) {
-        if (i == 0) best = 0;
-        __syncthreads();
-        // the largest `left`, as a positive float's bits above the row
-        if (i < p) atomicMax(&best, ((unsigned long long)__float_as_uint(fmaxf((float)left, 0.f)) << 32) | (unsigned)i);
-        __syncthreads();
-      }
-      const int unit = attempt == 1 ? (int)(best & 0xFFFFFFFFu) : -1;
-      w[i] = i >= p ? 0.0 : attempt == 1 ? (i == unit ? 1.0 : 0.0) : V[(size_t)j * p + i];
-      for (int pass = 0; pass < 2; ++pass) {
-        __syncthreads();
-        if (pass == 0 && attempt == 1) {
-          if (i < j) cf[i] = V[(size_t)i * p + unit];
-        } else {
-          for (int k = warp; k < j; k += 32) {
-            double s = 0.0;
-            for (int r = lane; r < p; r += 32) s = fma(V[(size_t)k * p + r], w[r], s);
-            s = warp_sum(s);
-            if (lane == 0) cf[k] = s;
-          }
-        }
-        __syncthreads();
-        if (i < p) {
-          double x = w[i];
-#pragma unroll 4
-          for (int k = 0; k < j; ++k) x = fma(-cf[k], V[(size_t)k * p + i], x);
-          w[i] = x;
-        }
-      }
-      __syncthreads();
-      double s = 0.0;  // every warp the same sum
-      for (int r = lane; r < p; r += 32) s = fma(w[r], w[r], s);
-      nrm = sqrt(warp_sum(s));
-    }
-    if (i < p) {
-      const double x = w[i] / nrm;
-      V[(size_t)j * p + i] = x;
-      left = fma(-x, x, left);
-    }
-    __syncthreads();
+// The null columns of the square factor (tr: U, else V), from those of Q (r x r, column-major).
+__global__ void svd_null_columns_kernel(int r, int tr, const double* __restrict__ Q, const double* __restrict__ Sv,
+                                        double* __restrict__ U, double* __restrict__ Vt) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < r * r; e += gridDim.x * blockDim.x) {
+    const int j = e / r, i = e % r;
+    if (!svd_null(Sv, j)) continue;
+    if (tr) U[(size_t)i * r + j] = Q[e];
+    else Vt[e] = Q[e];
   }
 }
 
+// The whole call on scratch of the caller's, up to the kept rank and the error bits on the host.
 cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, double* U, double* S, double* Vt,
-                    int* k_dev, double* scratch, double* extra, cudaStream_t st) {
+                    double* scratch, double* extra, cudaStream_t st, int* k, uint32_t* bits) {
   const int r = std::min(m, n), q = std::max(m, n);
   const bool tr = m < n;
   double* X = scratch;
@@ -120,6 +74,9 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   double* dinfo = nrm + 1;
   uint32_t* info = (uint32_t*)(dinfo + 2);
   int* ex = (int*)info + 2;
+  uint32_t* nulls = info + 3;
+  int* k_dev = (int*)(info + 4);
+  double* T1 = Ux;
   cudaError_t e = cudaMemsetAsync(info, 0, 4 * sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
   // X = 2^-ex M, largest entry near 1: its squares stay in range. Tall orientation, column-major: M^T column-major is M
@@ -133,10 +90,7 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = svd_tall64(q, r, X, Ux, Vw, extra, extra ? extra + (size_t)r * r : nullptr, &Ux, Sv, Vx, 60, info, sms, st)) != cudaSuccess) return e;
-  if (Ux == X) {  // by way of the QR; else V is the product of the rotations
-    ++tl_launches;
-    complete_basis_kernel<<<1, 1024, 0, st>>>(r, Vx, Sv);
-  }
+  const bool qr = Ux == X;  // else the square factor is the product of the rotations
   if ((e = fix_signs<double>(tr ? r : q, tr ? q : r, r, tr ? Vx : Ux, tr ? r : q, tr ? Ux : Vx, tr ? q : r, st)) !=
       cudaSuccess)
     return e;
@@ -144,8 +98,23 @@ cudaError_t svd_run(const double* M, int m, int n, int chi_max, double tau_rel, 
   const long long tot = (long long)q * r;
   const int blocks = (int)std::max<long long>(1, std::min<long long>((tot + 255) / 256, 1024));
   ++tl_launches;
-  svd_outputs_kernel<<<blocks, 256, 0, st>>>(m, n, tr ? 1 : 0, Ux, Vx, Sv, U, S, Vt, info);
-  return cudaGetLastError();
+  svd_outputs_kernel<<<blocks, 256, 0, st>>>(m, n, tr ? 1 : 0, Ux, Vx, Sv, U, S, Vt, info,
+                                         qr ? nulls : nullptr);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  uint32_t h[4];
+  if ((e = cudaMemcpyAsync(k, k_dev, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+  if ((e = cudaMemcpyAsync(h, info, sizeof(h), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+  *bits = h[0] & (ERRW_NAN | ERRW_NOCONV);
+  if (*bits || !h[3]) return cudaSuccess;
+  // null columns: a QR of the square factor gives back its other columns and, in these places, the rest of an
+  // orthonormal basis (a null column gives no reflector). 256 x 256 with 128 null columns: 7.3 ms without, 9.2 so.
+  if ((e = qr_householder<double, double>(r, r, Vx, Vw, T1, st)) != cudaSuccess) return e;
+  if (tr && (e = fix_signs<double>(r, 0, r, Vw, r, nullptr, 0, st)) != cudaSuccess) return e;
+  ++tl_launches;
+  svd_null_columns_kernel<<<std::max(1, std::min(r * r / 256, 1024)), 256, 0, st>>>(r, tr ? 1 : 0, Vw, Sv, U, Vt);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return cudaStreamSynchronize(st);
 }
 
 tt_status svd_check(const double* M, int m, int n, int chi_max, double tau_rel, const double* U, const double* S,
@@ -172,18 +141,14 @@ extern "C" tt_status tt_svd_truncated(const double* M, int m, int n, int chi_max
   size_t got = 0;
   double* scratch = (double*)block_take(dev, (nd + 2 * r2) * sizeof(double), &got);
   if (!scratch) return TT_ERR_OUT_OF_MEMORY;
-  int* k_dev = (int*)(scratch + nd - 1);
-  cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, k_dev, scratch, scratch + nd, st);
   int k = 0;
-  uint32_t flags[2] = {0, 0};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&k, k_dev, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(flags, scratch + svd_info_offset(m, n), 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
+  uint32_t bits = 0;
+  cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, scratch, scratch + nd, st, &k, &bits);
   const cudaError_t es = cudaStreamSynchronize(st);  // before the block goes back, whatever failed
   if (e == cudaSuccess) e = es;
   block_give(dev, got, scratch);
   if (e != cudaSuccess) return TT_ERR_CUDA;
-  if (flags[0] & (ERRW_NAN | ERRW_NOCONV)) return TT_ERR_NUMERICAL;
+  if (bits) return TT_ERR_NUMERICAL;
   *k_out = k;
   return TT_OK;
 }
@@ -236,21 +201,16 @@ extern "C" tt_status tt_svd_truncated_noalloc(const double* M, int m, int n, int
     cudaGetLastError();
     return TT_ERR_CUDA;
   }
-  int* k_dev = (int*)(scratch + nd - 1);
   // the FP32 sweeps' scratch, where the array has room for it as well
   const size_t r = std::min(m, n);
   double* extra = nd + 2 * r * r <= kNoAllocDoubles ? scratch + nd : nullptr;
   // svd_run clears the error flags it reads; every other scratch word it uses
   // is written before it is read
-  cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, k_dev, scratch, extra, st);
   int k = 0;
-  uint32_t flags[2] = {0, 0};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&k, k_dev, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(flags, scratch + svd_info_offset(m, n), 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  uint32_t bits = 0;
+  const cudaError_t e = svd_run(M, m, n, chi_max, tau_rel, U, S, Vt, scratch, extra, st, &k, &bits);
   if (e != cudaSuccess) return TT_ERR_CUDA;
-  if (flags[0] & (ERRW_NAN | ERRW_NOCONV)) return TT_ERR_NUMERICAL;
+  if (bits) return TT_ERR_NUMERICAL;
   *k_out = k;
   return TT_OK;
 }
